@@ -111,6 +111,12 @@ int cuda_fail(gal_ctx* ctx, cudaError_t e) {
     if (_e != cudaSuccess) return cuda_fail(ctx, _e); \
   } while (0)
 
+#define GAL_TRY(expr)            \
+  do {                           \
+    int _s = (expr);             \
+    if (_s != GAL_OK) return _s; \
+  } while (0)
+
 bool pow2_size(int n) { return n >= 4 && n <= (1 << kMaxLog2) && (n & (n - 1)) == 0; }
 int log2i(int n) {
   int l = 0;
@@ -144,6 +150,32 @@ cudaError_t grow(gal_ctx* ctx, void** p, size_t* have, size_t need) {
 
 template <typename T> constexpr int prec_index() { return sizeof(T) == 8 ? 1 : 0; }
 
+// the float table holds nxy complex values, the double one nxy more factors
+// of 16 bytes after them
+constexpr size_t twiddle_bytes(int nxy, bool f64) { return (size_t)nxy * (f64 ? 32 : 8); }
+template <typename T> constexpr size_t twiddle_bytes(int nxy) {
+  return twiddle_bytes(nxy, sizeof(T) == 8);
+}
+constexpr int kSinCosLen = 1024;
+
+// Twiddle table of length nxy (Launch::twiddles); in double the table of
+// length 1024 also serves the gather's sines and cosines.
+template <typename T> int ensure_twiddles(gal_ctx* ctx, int nxy) {
+  void*& tw = ctx->tw[prec_index<T>()][log2i(nxy)];
+  if (!tw) {
+    GAL_CUDA(ctx, cudaMalloc(&tw, twiddle_bytes<T>(nxy)));
+    ++g_ws_generation;
+    GAL_CUDA(ctx, gal::Launch<T>::twiddles(tw, nxy, 0));
+    GAL_CUDA(ctx, cudaStreamSynchronize(0));
+    ctx->launches++;
+  }
+  return GAL_OK;
+}
+template <typename T> int ensure_tables(gal_ctx* ctx, int nxy) {
+  GAL_TRY(ensure_twiddles<T>(ctx, nxy));
+  return sizeof(T) == 8 ? ensure_twiddles<T>(ctx, kSinCosLen) : GAL_OK;
+}
+
 // Workspace and twiddles for images of side nxy in precision T (full: the
 // full-plane path, whose row pass keeps up to nxy columns).
 template <typename T> int ensure(gal_ctx* ctx, int nxy, bool full = false) {
@@ -151,15 +183,7 @@ template <typename T> int ensure(gal_ctx* ctx, int nxy, bool full = false) {
   const size_t spec = (size_t)nxy * (nxy / 2 + 1) * sizeof(C);
   GAL_CUDA(ctx, grow(ctx, &ctx->F1, &ctx->F1_bytes, full ? (size_t)nxy * nxy * sizeof(C) : spec));
   GAL_CUDA(ctx, grow(ctx, &ctx->Gw, &ctx->Gw_bytes, 2 * spec));  // horizontal node pairs
-  const int l = log2i(nxy);
-  void*& tw = ctx->tw[prec_index<T>()][l];
-  if (!tw) {
-    GAL_CUDA(ctx, cudaMalloc(&tw, (size_t)nxy * sizeof(C)));
-    GAL_CUDA(ctx, gal::Launch<T>::twiddles(tw, nxy, 0));
-    GAL_CUDA(ctx, cudaStreamSynchronize(0));
-    ctx->launches++;
-  }
-  return GAL_OK;
+  return ensure_tables<T>(ctx, nxy);
 }
 
 cudaEvent_t pool_event(gal_ctx* ctx) {
@@ -214,12 +238,6 @@ template <typename F> int stage(gal_ctx* ctx, int id, cudaStream_t st, F&& launc
   return GAL_OK;
 }
 
-#define GAL_TRY(expr)            \
-  do {                           \
-    int _s = (expr);             \
-    if (_s != GAL_OK) return _s; \
-  } while (0)
-
 int check_geometry(int nxy, double dxy) {
   if (!pow2_size(nxy)) return GAL_E_INVAL;
   if (!(dxy > 0.0) || !std::isfinite(dxy)) return GAL_E_INVAL;
@@ -233,7 +251,7 @@ int check_profile(const void* I, int nr, double Rmin, double dR, double inc) {
   return GAL_OK;
 }
 
-gal::GatherParams gather_params(int nxy, double dxy, double dRA, double dDec, double PA) {
+gal::GatherParams gather_params(const gal_ctx* ctx, int nxy, double dxy, double dRA, double dDec, double PA) {
   gal::GatherParams g;
   g.cpa = std::cos(PA);
   g.spa = std::sin(PA);
@@ -241,6 +259,8 @@ gal::GatherParams gather_params(int nxy, double dxy, double dRA, double dDec, do
   g.phx = dRA;
   g.phy = dDec;
   g.N = nxy;
+  const char* t = static_cast<const char*>(ctx->tw[1][log2i(kSinCosLen)]);  // null until a double call
+  g.sincos = t ? t + 16 * kSinCosLen : nullptr;
   return g;
 }
 
@@ -429,7 +449,7 @@ int sample_impl(gal_ctx* ctx, const T* image, const T* I, const gal::SweepParams
   const T* beam;
   GAL_TRY(beam_tables<T>(ctx, o, nxy, dxy, dRA, dDec, PA, st, &beam));
   GAL_TRY(spectrum<T>(ctx, image, I, sp, nxy, dxy, ctx->rho2, 0, st, beam, o.full));
-  const gal::GatherParams gp = gather_params(nxy, dxy, dRA, dDec, PA);
+  const gal::GatherParams gp = gather_params(ctx, nxy, dxy, dRA, dDec, PA);
   if (o.full) {
     const int blocks = ctx->num_sms * gal::Plane<T>::gather_blocks_per_sm(false, 0);
     return stage(ctx, 3, st, [&] {
@@ -487,7 +507,7 @@ int chi2_impl(gal_ctx* ctx, const T* image, const T* I, const gal::SweepParams& 
   const gal::Bounds bd = gal::make_bounds(d->rho2_host, (double)nxy * dxy, nxy);
   const T* beam;
   GAL_TRY(beam_tables<T>(ctx, o, nxy, dxy, dRA, dDec, PA, st, &beam));
-  const gal::GatherParams gp = gather_params(nxy, dxy, dRA, dDec, PA);
+  const gal::GatherParams gp = gather_params(ctx, nxy, dxy, dRA, dDec, PA);
   if (o.full) {
     const int W = gal::full_cols(bd, nxy).W;
     GAL_TRY(spectrum<T>(ctx, image, I, sp, nxy, dxy, d->rho2, W, st, beam, true));
@@ -941,7 +961,8 @@ int plan_batch(gal_ctx* ctx, const gal_request* reqs, int n, double* chi2_out, B
     const gal::Bounds bd = gal::make_bounds(d->rho2_host, b.S, r.nxy);
     b.Kc = bd.Kc;
     b.nrw = bd.nrw;
-    b.gp = gather_params(r.nxy, r.dxy, r.dRA, r.dDec, r.PA);
+    if (p) GAL_TRY(ensure_twiddles<double>(ctx, kSinCosLen));
+    b.gp = gather_params(ctx, r.nxy, r.dxy, r.dRA, r.dDec, r.PA);
     b.u = d->u;
     b.v = d->v;
     b.re = d->re;
@@ -1003,19 +1024,6 @@ int plan_batch(gal_ctx* ctx, const gal_request* reqs, int n, double* chi2_out, B
       b.beam = offs[p][k].bm ? base + offs[p][k].bm : nullptr;
       b.counter = ctx->batch_ctr + reinterpret_cast<size_t>(b.counter);
     }
-  return GAL_OK;
-}
-
-template <typename T> int ensure_twiddles(gal_ctx* ctx, int nxy) {
-  using C = gal::cplx_t<T>;
-  void*& tw = ctx->tw[prec_index<T>()][log2i(nxy)];
-  if (!tw) {
-    GAL_CUDA(ctx, cudaMalloc(&tw, (size_t)nxy * sizeof(C)));
-    ++g_ws_generation;
-    GAL_CUDA(ctx, gal::Launch<T>::twiddles(tw, nxy, 0));
-    GAL_CUDA(ctx, cudaStreamSynchronize(0));
-    ctx->launches++;
-  }
   return GAL_OK;
 }
 
@@ -1150,8 +1158,8 @@ int run_batch(gal_ctx* ctx, const gal_request* reqs, int n, double* chi2_out, cu
   BatchPlan pl;
   GAL_TRY(plan_batch(ctx, reqs, n, chi2_out, pl));
   if (allow_setup) {
-    for (const auto& b : pl.items[0]) GAL_TRY(ensure_twiddles<float>(ctx, b.N));
-    for (const auto& b : pl.items[1]) GAL_TRY(ensure_twiddles<double>(ctx, b.N));
+    for (const auto& b : pl.items[0]) GAL_TRY(ensure_tables<float>(ctx, b.N));
+    for (const auto& b : pl.items[1]) GAL_TRY(ensure_tables<double>(ctx, b.N));
     for (const auto& b : pl.items[0]) GAL_TRY(fft_plan<float>(ctx, b.N, st));
   }
   // every request runs with the FFT plan of its side (the same as a single call's)
@@ -1375,7 +1383,7 @@ size_t gal_workspace_bytes(const gal_ctx* ctx) {
              (ctx->pipe_chi2 ? 2 * sizeof(double) : 0);
   for (int p = 0; p < 2; ++p)
     for (int l = 0; l <= kMaxLog2; ++l)
-      if (ctx->tw[p][l]) b += ((size_t)1 << l) * (p ? 16 : 8);
+      if (ctx->tw[p][l]) b += twiddle_bytes(1 << l, p == 1);
   return b;
 }
 
@@ -1490,8 +1498,8 @@ int gal_graph_launch(gal_graph* g, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     BatchPlan pl;
     GAL_TRY(plan_batch(ctx, g->reqs.data(), (int)g->reqs.size(), g->chi2_out, pl));
-    for (const auto& b : pl.items[0]) GAL_TRY(ensure_twiddles<float>(ctx, b.N));
-    for (const auto& b : pl.items[1]) GAL_TRY(ensure_twiddles<double>(ctx, b.N));
+    for (const auto& b : pl.items[0]) GAL_TRY(ensure_tables<float>(ctx, b.N));
+    for (const auto& b : pl.items[1]) GAL_TRY(ensure_tables<double>(ctx, b.N));
     for (int i : pl.single) {
       const gal_request& r = g->reqs[i];
       GAL_TRY(r.data->real_bytes == 8 ? ensure<double>(ctx, r.nxy) : ensure<float>(ctx, r.nxy));

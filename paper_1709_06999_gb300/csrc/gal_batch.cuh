@@ -43,7 +43,9 @@ cudaError_t rows(const BatchItem* it, const int* idx, int n, const void* tw, int
                         b.S, BEAM ? static_cast<const T*>(b.beam) : nullptr};
   }
   const C* twc = static_cast<const C*>(tw);
-  if constexpr (row_ldg_shape<T, LG, SWEEP, V>()) {
+  if constexpr (sizeof(T) == 8) {
+    return launch_row_fx<LG, SWEEP, kBatchJobs, BEAM>(jb, n, sh.row_blocks, false, twc, err, st);
+  } else if constexpr (row_ldg_shape<T, LG, SWEEP, V>()) {
     // the same kernel as single calls of this length (bitwise equal results)
     constexpr auto kern = row_fft3_ldg_kernel<kBatchJobs, BEAM>;
     const cudaError_t e = ensure_smem_attr<kern>(RowLdgShape::smem);
@@ -99,11 +101,6 @@ template <typename T, int LG, int V = FftV<T>::V>
 cudaError_t cols(const BatchItem* it, const int* idx, int n, const void* tw, cudaStream_t st) {
   using C = cplx_t<T>;
   constexpr int N = 1 << LG;
-  using SH = ColShape3<T, N, V>;
-  constexpr auto kern = col_fft3_kernel<T, LG, kBatchJobs, V>;
-  const size_t smem = (size_t)2 * SH::G * SH::RS * sizeof(C);
-  const cudaError_t e = ensure_smem_attr<kern>(smem);
-  if (e) return e;
   Jobs<ColJob<T>, kBatchJobs> jb{};
   int kc = 1;
   for (int k = 0; k < n; ++k) {
@@ -112,11 +109,20 @@ cudaError_t cols(const BatchItem* it, const int* idx, int n, const void* tw, cud
                         b.full ? 1 : 0};
     kc = b.ncol > kc ? b.ncol : kc;
   }
-  int x = (kc + SH::G - 1) / SH::G;
-  const int cap = 2 * current_device_sms();
-  if (x > cap) x = cap;
-  kern<<<dim3(x, n), SH::threads, smem, st>>>(jb, static_cast<const C*>(tw));
-  return cudaGetLastError();
+  if constexpr (sizeof(T) == 8) {
+    return launch_col_fx<LG, kBatchJobs>(jb, n, kc, false, static_cast<const C*>(tw), st);
+  } else {
+    using SH = ColShape3<T, N, V>;
+    constexpr auto kern = col_fft3_kernel<T, LG, kBatchJobs, V>;
+    const size_t smem = (size_t)2 * SH::G * SH::RS * sizeof(C);
+    const cudaError_t e = ensure_smem_attr<kern>(smem);
+    if (e) return e;
+    int x = (kc + SH::G - 1) / SH::G;
+    const int cap = 2 * current_device_sms();
+    if (x > cap) x = cap;
+    kern<<<dim3(x, n), SH::threads, smem, st>>>(jb, static_cast<const C*>(tw));
+    return cudaGetLastError();
+  }
 }
 
 // Each request keeps the block partition of its single call (`grid` virtual

@@ -15,6 +15,11 @@ template <typename T> using cplx_t = typename cplx<T>::type;
 
 __host__ __device__ __forceinline__ float2 mkc(float x, float y) { return make_float2(x, y); }
 __host__ __device__ __forceinline__ double2 mkc(double x, double y) { return make_double2(x, y); }
+// 64-bit fixed-point complex value (gal_fx.cuh)
+struct fx2 {
+  long long x, y;
+};
+__host__ __device__ __forceinline__ fx2 mkc(long long x, long long y) { return fx2{x, y}; }
 
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return mkc(a.x + b.x, a.y + b.y); }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return mkc(a.x - b.x, a.y - b.y); }

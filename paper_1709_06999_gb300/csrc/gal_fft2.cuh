@@ -25,16 +25,19 @@ template <typename C> __device__ __forceinline__ void bfly4(C& a0, C& a1, C& a2,
   a3 = csub(d2, d3);
 }
 
+// x / sqrt 2
+template <typename R> __device__ __forceinline__ R mul_sqrt_half(R x) {
+  return x * (R)0.70710678118654752440084436210484903928;
+}
+
 template <typename C> __device__ __forceinline__ void bfly8(C* a) {
-  using R = decltype(a[0].x);
-  const R h = (R)0.70710678118654752440084436210484903928;
   C b0 = cadd(a[0], a[4]), b4 = csub(a[0], a[4]);
   C b1 = cadd(a[1], a[5]), b5 = csub(a[1], a[5]);
   C b2 = cadd(a[2], a[6]), b6 = csub(a[2], a[6]);
   C b3 = cadd(a[3], a[7]), b7 = csub(a[3], a[7]);
-  b5 = mkc((b5.x + b5.y) * h, (b5.y - b5.x) * h);
+  b5 = mkc(mul_sqrt_half(b5.x + b5.y), mul_sqrt_half(b5.y - b5.x));
   b6 = cmul_mi(b6);
-  b7 = mkc((b7.y - b7.x) * h, -(b7.x + b7.y) * h);
+  b7 = mkc(mul_sqrt_half(b7.y - b7.x), mul_sqrt_half(-(b7.x + b7.y)));
   bfly4(b0, b1, b2, b3);
   bfly4(b4, b5, b6, b7);
   a[0] = b0; a[2] = b1; a[4] = b2; a[6] = b3;

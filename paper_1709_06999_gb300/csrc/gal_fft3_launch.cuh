@@ -4,6 +4,7 @@
 
 #include <type_traits>
 
+#include "gal_fx_kernels.cuh"
 #include "gal_kernels.cuh"
 
 namespace gal {
@@ -32,7 +33,9 @@ cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc,
                              cudaStream_t st) {
   using C = cplx_t<T>;
   constexpr int M = 1 << LG, N = 2 * M;
-  if constexpr (row_ldg_shape<T, LG, SWEEP, V>()) {  // float rows of 4096 pixels
+  if constexpr (sizeof(T) == 8) {  // double rows: on integers
+    return launch_row_fx<LG, SWEEP, 1, BEAM>(jb, 1, 1, BEAM, twc, err, st);
+  } else if constexpr (row_ldg_shape<T, LG, SWEEP, V>()) {  // float rows of 4096 pixels
     constexpr auto kern = row_fft3_ldg_kernel<1, BEAM>;
     cudaError_t e = ensure_smem_attr<kern>(RowLdgShape::smem);
     if (e) return e;
@@ -92,20 +95,24 @@ cudaError_t launch_col3_kern(const void* F1, void* Gw, const void* tw, const dou
                              int kc_hint, bool full, cudaStream_t st) {
   using C = cplx_t<T>;
   constexpr int N = 1 << LG;
-  using SH = ColShape3<T, N, V>;
-  constexpr auto kern = col_fft3_kernel<T, LG, 1, V>;
-  const size_t smem = (size_t)2 * SH::G * SH::RS * sizeof(C);
-  const cudaError_t e = ensure_smem_attr<kern>(smem);
-  if (e) return e;
   const int P = full ? N : N / 2 + 1;  // most window columns
   const int kc = kc_hint > 0 && kc_hint <= P ? kc_hint : P;
-  int col_blocks = (kc + SH::G - 1) / SH::G;
-  const int cap = 2 * current_device_sms();
-  if (col_blocks > cap) col_blocks = cap;
   Jobs<ColJob<T>, 1> jb;
   jb.j[0] = ColJob<T>{static_cast<const C*>(F1), static_cast<C*>(Gw), rho2, S, full ? 1 : 0};
-  return launch_dependent(kern, dim3(col_blocks), dim3(SH::threads), smem, st, jb,
-                          static_cast<const C*>(tw));
+  if constexpr (sizeof(T) == 8) {  // double columns: on integers
+    return launch_col_fx<LG, 1>(jb, 1, kc, true, static_cast<const C*>(tw), st);
+  } else {
+    using SH = ColShape3<T, N, V>;
+    constexpr auto kern = col_fft3_kernel<T, LG, 1, V>;
+    const size_t smem = (size_t)2 * SH::G * SH::RS * sizeof(C);
+    const cudaError_t e = ensure_smem_attr<kern>(smem);
+    if (e) return e;
+    int col_blocks = (kc + SH::G - 1) / SH::G;
+    const int cap = 2 * current_device_sms();
+    if (col_blocks > cap) col_blocks = cap;
+    return launch_dependent(kern, dim3(col_blocks), dim3(SH::threads), smem, st, jb,
+                            static_cast<const C*>(tw));
+  }
 }
 
 template <typename T, int LG>

@@ -15,6 +15,7 @@
 #include "gal_fft.cuh"
 #include "gal_fft2.cuh"
 #include "gal_fft3.cuh"
+#include "gal_fx.cuh"
 #include "gal_tma.cuh"
 
 #include <atomic>
@@ -35,6 +36,8 @@ __global__ void twiddle_kernel(cplx_t<T>* __restrict__ tw, int N) {
   double s, c;
   sincospi(-2.0 * (double)k / (double)N, &s, &c);
   tw[k] = mkc((T)c, (T)s);
+  // the double table is followed by the same factors for the integer passes
+  if constexpr (sizeof(T) == 8) reinterpret_cast<fxtw*>(tw + N)[k] = fx_factor(c, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -898,14 +901,15 @@ template <typename T> struct ColJob {
 };
 
 template <> struct GatherT<double> {
-  double cpa, spa, S, phx, phy;
+  double A, B, phx, phy;  // A = cos(PA) N dxy, B = sin(PA) N dxy, as for float
   double Sd;
+  const fxtw* sincos;     // factors W_1024^k (kSinCos of them)
   int N;
   __host__ static GatherT make(const GatherParams& g) {
     GatherT r;
-    r.cpa = g.cpa;
-    r.spa = g.spa;
-    r.S = g.S;
+    r.A = g.cpa * g.S;
+    r.B = g.spa * g.S;
+    r.sincos = static_cast<const fxtw*>(g.sincos);
     r.phx = g.phx;
     r.phy = g.phy;
     r.Sd = g.S;
@@ -1331,62 +1335,74 @@ __device__ __forceinline__ void sample_pair(const float2* __restrict__ G, const 
   V1 = fma2(pk(s1, s1), pk(-A1.y, A1.x), mul2(pk(c1, c1), A1));
 }
 
-// cell of the position ofs + x (x relative to the window's origin row or
-// column ofs), clamped to the window's node range [0, last + 1].  The floor
-// is taken of x itself so the result does not depend on the window's size.
-__device__ __forceinline__ void cell_d(double x, int ofs, int last, int& c, double& f) {
-  double fl = floor(x);
-  f = x - fl;
-  fl = fmin(fmax(fl, -1.0e9), 1.0e9);
-  c = (int)fl + ofs;
-  if (c < 0) {
-    c = 0;
-    f = 0.0;
-  } else if (c > last) {
-    c = last;
-    f = 1.0;
-  }
-}
-
+// double path: FP64 for the rotation and the phase argument, integers (gal_fx.cuh)
+// for the cell, the interpolation, the sine and cosine and the phase rotation:
+// about 17 FP64 instructions a point instead of about 95, which bounded this
+// kernel (5e6 points, window in shared memory: 726 -> 181 us; 1e6 points, window
+// through L2: 155 -> 48 us).  tab: the sine / cosine table in shared memory.
 template <bool SMEM, bool EDGE, bool MULTI = false, bool FULL = false>
 __device__ __forceinline__ double2 sample_point(const cplx_t<double>* __restrict__ Gp, const Window& w,
                                                 const GatherT<double>& p, double u, double v,
-                                                const MultiPhase<double>* mp = nullptr) {
-  if (!(isfinite(u) && isfinite(v)))
-    return make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
-  double up = u * p.cpa - v * p.spa;
-  double vp = u * p.spa + v * p.cpa;
-  const bool neg = !FULL && up < 0.0;  // Hermitian fold (half spectrum only)
+                                                const MultiPhase<double>* mp, const fxtw* tab) {
+  const double x = u * p.A - v * p.B, y = u * p.B + v * p.A;
+  bool bad = fx_isnan(x) || fx_isnan(y);
+  long long xf = fx_pos(x), yf = fx_pos(y);
+  const bool neg = !FULL && __double2hiint(x) < 0 &&
+                   (fx_ebits(x) | (unsigned)__double2loint(x)) != 0u;  // x < 0: Hermitian fold
   if (neg) {
-    up = -up;
-    vp = -vp;
+    xf = -xf;
+    yf = -yf;
   }
-  int r, c;
-  double fr, fc;
-  cell_d(vp * p.S, w.rofs, w.rmax, r, fr);
-  cell_d(up * p.S, FULL ? w.cofs : 0, w.cmax, c, fc);
+  // cell and fraction, clamped to the node range
+  auto cell = [](long long f, int ofs, int last, int& c, int& fh, int& fl) {
+    c = (int)(f >> kPosBits) + ofs;
+    long long t = (f & ((1ll << kPosBits) - 1)) << (62 - kPosBits);
+    if (c < 0) {
+      c = 0;
+      t = 0;
+    } else if (c > last) {
+      c = last;
+      t = 1ll << 62;
+    }
+    fx_split(t, fh, fl);
+  };
+  int c, r, cfh, cfl, rfh, rfl;
+  cell(yf, w.rofs, w.rmax, r, rfh, rfl);
+  cell(xf, FULL ? w.cofs : 0, w.cmax, c, cfh, cfl);
   const double2* g = Gp + (size_t)r * w.pitch + c;
   const double2 g00 = ld_node<SMEM>(g), g01 = ld_node<SMEM>(g + 1);
   const double2 g10 = ld_node<SMEM>(g + w.pitch), g11 = ld_node<SMEM>(g + w.pitch + 1);
-  double2 V = clerp(clerp(g00, g01, fc), clerp(g10, g11, fc), fr);
+  const unsigned h = max(max(max(fx_ebits(g00.x), fx_ebits(g00.y)), max(fx_ebits(g01.x), fx_ebits(g01.y))),
+                         max(max(fx_ebits(g10.x), fx_ebits(g10.y)), max(fx_ebits(g11.x), fx_ebits(g11.y))));
+  const int E = max((int)(h >> 20), 1);
+  bad = bad || E >= 0x7ff;
+  auto node = [&](double2 a) { return fx2{fx_node(a.x, E), fx_node(a.y, E)}; };
+  fx2 V = fx_lerp(fx_lerp(node(g00), node(g01), cfh, cfl), fx_lerp(node(g10), node(g11), cfh, cfl), rfh, rfl);
   if (neg) V.y = -V.y;
-  double sn, cs;
-  if constexpr (MULTI) {
-    cs = 0.0;
-    sn = 0.0;
+  const int q = E - 1082;
+  // V turned by one offset's phase
+  auto turned = [&](double phx, double phy) {
+    const double ph = u * phx + v * phy;
+    bad = bad || fx_nonfinite(ph);
+    const fx2 e = fx_cos_sin(fx_turns(ph), tab);
+    fxtw f;
+    fx_digits(e.x, f.xh, f.xl);
+    fx_digits(e.y, f.yh, f.yl);
+    const fx2 R = cmul(V, f);
+    return make_double2(fx_to(R.x, q), fx_to(R.y, q));
+  };
+  double2 out;
+  if constexpr (MULTI) {  // (one copy of amplitude 1 is the single call, bit for bit)
+    out = make_double2(0.0, 0.0);
     for (int k = 0; k < mp->K; ++k) {
-      const double ph = u * mp->phx[k] + v * mp->phy[k];
-      double sk, ck;
-      sincospi(2.0 * (ph - rint(ph)), &sk, &ck);
-      cs = fma(mp->amp[k], ck, cs);
-      sn = fma(mp->amp[k], sk, sn);
+      const double2 R = turned(mp->phx[k], mp->phy[k]);
+      out.x = fma(mp->amp[k], R.x, out.x);
+      out.y = fma(mp->amp[k], R.y, out.y);
     }
   } else {
-    const double ph = u * p.phx + v * p.phy;
-    const double fph = ph - rint(ph);
-    sincospi(2.0 * fph, &sn, &cs);
+    out = turned(p.phx, p.phy);
   }
-  return cmul(V, make_double2(cs, sn));
+  return bad ? make_double2(fx_nan(), fx_nan()) : out;
 }
 
 // per-thread compensated accumulators
@@ -1441,7 +1457,10 @@ struct AccD {  // Neumaier
   double s = 0.0, c = 0.0;
   __device__ __forceinline__ void add(double x) {
     const double t = s + x;
-    c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
+    // the larger exponent first (bits order like the exponent; equal ones go either way)
+    const bool big = fx_ebits(s) >= fx_ebits(x);
+    const double a = big ? s : x, b = big ? x : s;
+    c += (a - t) + b;
     s = t;
   }
   __device__ __forceinline__ double value() const { return s + c; }
@@ -1534,11 +1553,13 @@ __device__ __forceinline__ void gather_points(const cplx_t<T>* __restrict__ G, c
                                               const T* __restrict__ im, const T* __restrict__ w,
                                               int64_t M, int vec, cplx_t<T>* __restrict__ vis,
                                               ACC& acc, const MultiPhase<T>* mp,
-                                              const PointGroup<T, CHI2>* pre, const GroupSplit& sp) {
+                                              const PointGroup<T, CHI2>* pre, const GroupSplit& sp,
+                                              const fxtw* tab) {
   using C = cplx_t<T>;
   constexpr int W = Vec16<T>::W;
   auto point = [&](T uu, T vv) {
-    return sample_point<SMEM, EDGE, MULTI, FULL>(G, win, p, uu, vv, mp);
+    if constexpr (sizeof(T) == 8) return sample_point<SMEM, EDGE, MULTI, FULL>(G, win, p, uu, vv, mp, tab);
+    else return sample_point<SMEM, EDGE, MULTI, FULL>(G, win, p, uu, vv, mp);
   };
   const int64_t gtid = sp.gtid;
   auto compute = [&](const PointGroup<T, CHI2>& g, int64_t q) {  // the W points of group q
@@ -1655,6 +1676,13 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
       }
     }
   }
+  const fxtw* tab = nullptr;
+  if constexpr (sizeof(T) == 8) {
+    __shared__ fxtw sct[kSinCos];  // read by every point at a random place: shared memory, 16 KB
+    for (int i = threadIdx.x; i < kSinCos; i += blockDim.x) sct[i] = ldg_tw(p.sincos + i);
+    __syncthreads();
+    tab = sct;
+  }
   grid_dep_wait();  // the window is the column pass's output
   C* sw = nullptr;
   bool win_ok = true;
@@ -1690,7 +1718,7 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
     if constexpr (SMEM) {
       if (win_ok) {
         gather_points<T, CHI2, true, EDGE, MULTI, FULL>(sw, win, p, u, v, re, im, w, M, vec, vis,
-                                                        acc, mp, g0p, sp);
+                                                        acc, mp, g0p, sp, tab);
       } else {
         const T nan = std::numeric_limits<T>::quiet_NaN();
         if constexpr (CHI2) {
@@ -1701,7 +1729,7 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
       }
     } else {
       gather_points<T, CHI2, false, EDGE, MULTI, FULL>(Gw, win, p, u, v, re, im, w, M, vec, vis,
-                                                       acc, mp, g0p, sp);
+                                                       acc, mp, g0p, sp, tab);
     }
     if constexpr (CHI2) {
       const double bs = acc.block_total(ws);
@@ -1755,7 +1783,7 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
 template <auto Kern> cudaError_t ensure_smem_attr(size_t smem) {
   constexpr int kDev = 64;
   static std::atomic<size_t> done[kDev] = {};
-  if (smem <= 48 * 1024) return cudaSuccess;
+  if (smem <= 24 * 1024) return cudaSuccess;  // with at most 24 KB static, below the default 48 KB
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e) return e;
