@@ -152,7 +152,7 @@ cudaError_t gather(const BatchItem* it, const int* idx, int n, int grid, int fol
   constexpr auto kern = gather_kernel<T, true, SMEM, EDGE, kBatchJobs, false, FULL>;
   const cudaError_t e = ensure_smem_attr<kern>(smem);
   if (e) return e;
-  const int threads = gather_threads<SMEM, FULL>();
+  const int threads = gather_threads<T, SMEM, FULL>();
   if (fold_max < 1) fold_max = 1;
   if (fold_max > kMaxGatherFold) fold_max = kMaxGatherFold;
   const int fold = n < fold_max ? n : fold_max;

@@ -3,7 +3,7 @@
 // common power of two before its transform.  Images, F1 and the window are
 // doubles.  Measured against the same passes in FP64 arithmetic (which kept the
 // FP64 pipe 83 % busy): row pass of 4096^2 pixels, 61 columns kept, 481 -> 113
-// us; of 2048^2 pixels, 413 columns kept, 161 -> 38 us; column pass of 4096 x 61
+// us (now 100); of 2048^2 pixels, 413 columns kept, 161 -> 38 us; column pass of 4096 x 61
 // 41 -> 12 us, of 2048 x 413 66 -> 19 us.
 #pragma once
 
@@ -14,21 +14,32 @@
 
 namespace gal {
 
-// Rows of 2^(LG+1) pixels as complex sequences of M = 2^LG points.
+// Rows of 2^(LG+1) pixels as complex sequences of M = 2^LG points, G rows to a
+// block of at least 128 threads.  One buffer of arriving rows beside the two
+// work buffers, not a ring of two that double as work buffers, lets two blocks
+// of 4096-pixel rows share an SM (116 KB each): 113 -> 100 us.  (Two rows of
+// 2048 pixels to a block of 256 threads: 1 % slower than one to 128.)
 template <int LG> struct FxRowShape {
   static constexpr int M = 1 << LG, N = 2 * M;
   using SH = Shape3<double, M, N, 128, 8>;
+  static constexpr int G = SH::G;
+  // row stride of the work buffers: half a bank row off, so that two rows read
+  // side by side do not collide
+  static constexpr int RS = SH::RS + (G > 1 ? 4 : 0);
   static constexpr int ntab = FxPlan<M>::ntab;
-  // header (barriers, reduction scratch, row scales), factor table, row buffers
+  // header (barrier, reduction scratch, row scales), factor table, two work
+  // buffers, the image rows as they arrive
   static constexpr int kHead = 512;
-  static constexpr size_t smem(bool tma) {
-    return kHead + (size_t)ntab * sizeof(fxtw) + (size_t)(tma ? 3 : 2) * SH::G * SH::RS * sizeof(fx2);
+  static constexpr size_t work = (size_t)G * RS * sizeof(fx2);
+  static constexpr size_t smem(bool image) {
+    return kHead + (size_t)ntab * sizeof(fxtw) + 2 * work + (image ? (size_t)G * N * sizeof(double) : 0);
   }
 };
 
-// Row pass (see row_fft3_kernel).  Persistent blocks own row groups; TMA: the
-// image rows come through a two-slot ring of bulk copies, SWEEP: they are
-// generated from the profile.
+// Row pass (see row_fft3_kernel).  Persistent blocks own row groups.  Image
+// rows come by bulk copy into a buffer of their own, which is free again as
+// soon as the rows are in registers, so the next group is in flight during the
+// whole transform; SWEEP: the rows are generated from the profile.
 template <int LG, bool SWEEP, int K, bool BEAM = false>
 __global__ void __launch_bounds__(FxRowShape<LG>::SH::threads,
                                   min_blocks_128regs<FxRowShape<LG>::SH::threads>())
@@ -38,61 +49,49 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
   using S = FxRowShape<LG>;
   using SH = typename S::SH;
   using P = typename SH::P;
-  constexpr int M = S::M, N = S::N, TT = P::T, G = SH::G, RS = SH::RS;
+  constexpr int M = S::M, N = S::N, TT = P::T, G = S::G, RS = S::RS;
   const RowJob<double>& jb = jobs.j[K == 1 ? 0 : blockIdx.y];
   const double* __restrict__ image = jb.image;
   const double* __restrict__ beam = BEAM ? jb.beam : nullptr;
   double2* __restrict__ F1 = jb.F1;
   const fxtw* __restrict__ tw = reinterpret_cast<const fxtw*>(twd + N);
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   unsigned* red_max = reinterpret_cast<unsigned*>(smem_raw + 32);   // one per warp, <= 16
   unsigned* red_sum = reinterpret_cast<unsigned*>(smem_raw + 96);
   int* row_q = reinterpret_cast<int*>(smem_raw + 192);              // per row of the group, <= 64
   fxtw* tab = reinterpret_cast<fxtw*>(smem_raw + S::kHead);
-  fx2* base = reinterpret_cast<fx2*>(smem_raw + S::kHead + (size_t)S::ntab * sizeof(fxtw));
+  fx2* A0 = reinterpret_cast<fx2*>(smem_raw + S::kHead + (size_t)S::ntab * sizeof(fxtw));
+  fx2* B0 = A0 + G * RS;
+  double* slot = reinterpret_cast<double*>(B0 + G * RS);
   static_assert(G <= 64 && SH::threads <= 512, "header");
   const int g = threadIdx.x / TT, t = threadIdx.x - g * TT;
   const int ngroups = N / G;
-  fx2* slot0 = base;
-  fx2* work = base + (size_t)(SWEEP ? 1 : 2) * G * RS;
   const uint32_t half_bytes = (uint32_t)(M * sizeof(double));
-  if constexpr (!SWEEP) {
-    if (threadIdx.x == 0) {
-      mbar_init(&bars[0], 1);
-      mbar_init(&bars[1], 1);
-      mbar_init_fence();
-    }
-    __syncthreads();
-  }
-  auto issue = [&](int it) {  // thread 0 only
-    const int grp = blockIdx.x + it * gridDim.x;
+  auto issue = [&](int grp) {  // thread 0 only
     if (grp >= ngroups) return;
-    const int sl = it & 1;
-    mbar_arrive_expect_tx(&bars[sl], 2u * half_bytes * (uint32_t)G);
+    mbar_arrive_expect_tx(bar, 2u * half_bytes * (uint32_t)G);
     for (int rl = 0; rl < G; ++rl) {
       const double* src = image + (size_t)(((grp * G + rl) + M) & (N - 1)) * N;
-      double* dst = reinterpret_cast<double*>(slot0 + (size_t)(sl * G + rl) * RS);
-      bulk_load(dst, src + M, half_bytes, &bars[sl]);
-      bulk_load(dst + M, src, half_bytes, &bars[sl]);
+      double* dst = slot + (size_t)rl * N;
+      bulk_load(dst, src + M, half_bytes, bar);
+      bulk_load(dst + M, src, half_bytes, bar);
     }
   };
   if constexpr (!SWEEP) {
     if (threadIdx.x == 0) {
-      issue(0);
-      issue(1);
+      mbar_init(bar, 1);
+      mbar_init_fence();
+      issue(blockIdx.x);
     }
   }
   fx_fill_tab<M, 2>(tab, tw);
   const Bounds bd = block_bounds(jb.rho2, jb.S, N);  // synchronises
   const bool pruned = P::nstage >= 2 && bd.Kc <= P::Nsl;
   if constexpr (BEAM) grid_dep_wait();  // the beam tables
-  for (int it = 0;; ++it) {
-    const int grp = blockIdx.x + it * gridDim.x;
-    if (grp >= ngroups) break;
-    const int sl = SWEEP ? 0 : it & 1;
+  uint32_t phase = 0;
+  for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x, phase ^= 1u) {
     const int row = grp * G + g;
-    fx2* slot = slot0 + (size_t)(sl * G + g) * RS;
     double2 z[8];
     if constexpr (SWEEP) {
       const int irow = (row + M) & (N - 1);
@@ -102,17 +101,23 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
         z[r] = make_double2(sweep_pixel(jb.I, jb.sp, N, irow, j), sweep_pixel(jb.I, jb.sp, N, irow, j + 1));
       }
     } else {
-      const bool ok = mbar_wait(&bars[sl], (uint32_t)((it >> 1) & 1));
+      // a wait that gives up (never expected) is reported, and the block ends:
+      // its one copy in flight is the one it has waited for
+      const bool ok = mbar_wait(bar, phase);
       if (__syncthreads_or(!ok)) {
         if (threadIdx.x == 0) {
           atomicOr(err, 2);
-          for (int k = it; k < it + 2; ++k)
-            if (blockIdx.x + k * gridDim.x < ngroups) mbar_wait(&bars[k & 1], (uint32_t)((k >> 1) & 1));
+          mbar_wait(bar, phase);
         }
         return;
       }
 #pragma unroll
-      for (int r = 0; r < 8; ++r) z[r] = reinterpret_cast<const double2*>(slot)[t + r * TT];
+      for (int r = 0; r < 8; ++r) z[r] = reinterpret_cast<const double2*>(slot + (size_t)g * N)[t + r * TT];
+      __syncthreads();  // the rows are in registers: the next group may land
+      if (threadIdx.x == 0) {
+        fence_proxy_async_smem();
+        issue(grp + gridDim.x);
+      }
     }
     if constexpr (BEAM) {
 #pragma unroll
@@ -120,45 +125,37 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
     }
     fx2 v[8];
     const FxScale sc = fx_load<TT>(z, v, red_max, red_sum);
-    // the slot is written from stage 1 on, after the barrier that ends stage 0
-    fx2* A = work + (size_t)g * RS;
-    fx2* B = slot;
+    if (t == 0) row_q[g] = sc.bad ? INT_MAX : sc.q;
+    fx2* A = A0 + g * RS;
+    fx2* B = B0 + g * RS;
     FxHead<M, 0>::run(v, A, B, t, tab);
     fx2* in = last_input<M, 8>(A, B);
-    double2* out = F1 + row;  // column-major: bin j of this row at out[j N]
-    auto emit = [&](double2* o, fx2 x2, int q, bool bad) {
-      *o = bad ? make_double2(fx_nan(), fx_nan()) : make_double2(fx_to(x2.x, q - 1), fx_to(x2.y, q - 1));
-    };
-    if (pruned) {
-      for (int j = t; j < bd.Kc; j += TT) {
-        fx2 zj, zmj;
-        fx_pruned_pair<M, 2>(in, j, tw, zj, zmj);
-        emit(out + (size_t)j * N, fx_r2c_unpack2(zj, zmj, ldg_tw(tw + j)), sc.q, sc.bad);
-      }
-    } else {
+    if (!pruned) {
       fx_last_full<M, 2>(v, in, t, tw);
-      fx2* o = in == A ? B : A;
-      store_full<M, 8>(v, o, t);
-      if (t == 0) row_q[g] = sc.bad ? INT_MAX : sc.q;
+      in = in == A ? B : A;
+      store_full<M, 8>(v, in, t);
       __syncthreads();
-      // bin by bin, the G rows of the group side by side (row_fft3_kernel)
-      const fx2* o0 = o - (size_t)g * RS;
-      double2* out0 = out - g;
-      for (int q = threadIdx.x; q < bd.Kc * G; q += G * TT) {
-        const int k = q / G, gg = q - k * G;
-        const fx2* og = o0 + (size_t)gg * RS;
-        emit(out0 + (size_t)k * N + gg,
-             fx_r2c_unpack2(og[pad3<8>(k & (M - 1))], og[pad3<8>((M - k) & (M - 1))], ldg_tw(tw + k)),
-             row_q[gg], row_q[gg] == INT_MAX);
-      }
     }
-    __syncthreads();  // every read of this slot and of the work buffer is done
-    if constexpr (!SWEEP) {
-      if (threadIdx.x == 0) {
-        fence_proxy_async_smem();
-        issue(it + 2);
+    // Bin by bin with the G rows of the group side by side, so that neighbouring
+    // lanes fill the sectors of a column of F1 (column-major: bin k of row i at
+    // F1[k N + i]); row gg's buffer lies (gg - g) RS from ours.
+    const fx2* in0 = in - g * RS;
+    for (int o = threadIdx.x; o < bd.Kc * G; o += G * TT) {
+      const int k = o / G, gg = o - k * G;
+      const fx2* x = in0 + gg * RS;
+      fx2 zk, zmk;
+      if (pruned) {
+        fx_pruned_pair<M, 2>(x, k, tw, zk, zmk);
+      } else {
+        zk = x[pad3<8>(k & (M - 1))];
+        zmk = x[pad3<8>((M - k) & (M - 1))];
       }
+      const fx2 X2 = fx_r2c_unpack2(zk, zmk, ldg_tw(tw + k));
+      const int q = row_q[gg];
+      F1[(size_t)k * N + grp * G + gg] =
+          q == INT_MAX ? make_double2(fx_nan(), fx_nan()) : make_double2(fx_to(X2.x, q - 1), fx_to(X2.y, q - 1));
     }
+    __syncthreads();  // every read of the work buffers and scales is done
   }
 }
 

@@ -1338,7 +1338,7 @@ __device__ __forceinline__ void sample_pair(const float2* __restrict__ G, const 
 // double path: FP64 for the rotation and the phase argument, integers (gal_fx.cuh)
 // for the cell, the interpolation, the sine and cosine and the phase rotation:
 // about 17 FP64 instructions a point instead of about 95, which bounded this
-// kernel (5e6 points, window in shared memory: 726 -> 181 us; 1e6 points, window
+// kernel (5e6 points, window in shared memory: 726 -> 168 us; 1e6 points, window
 // through L2: 155 -> 48 us).  tab: the sine / cosine table in shared memory.
 template <bool SMEM, bool EDGE, bool MULTI = false, bool FULL = false>
 __device__ __forceinline__ double2 sample_point(const cplx_t<double>* __restrict__ Gp, const Window& w,
@@ -1621,13 +1621,17 @@ __device__ __forceinline__ void gather_points(const cplx_t<T>* __restrict__ G, c
 // final reduction overlap the other's stream), 256-thread blocks otherwise.
 // The full-plane window is about twice as large, so only one copy fits per
 // SM: one 1024-thread block then keeps the same 32 warps resident.
-template <bool SMEM, bool FULL = false> constexpr int gather_threads() {
-  return SMEM ? (FULL ? 1024 : 512) : 256;
+// So is a double window, which the sine / cosine table accompanies (5e6 points,
+// 118 KB window: 181 us with one 512-thread block per SM, 168 us with 1024).
+template <typename T, bool SMEM, bool FULL = false> constexpr int gather_threads() {
+  return SMEM ? (FULL || sizeof(T) == 8 ? 1024 : 512) : 256;
 }
-template <bool SMEM, bool FULL> constexpr int gather_min_blocks() { return SMEM ? (FULL ? 1 : 2) : 4; }
+template <typename T, bool SMEM, bool FULL> constexpr int gather_min_blocks() {
+  return SMEM ? 1024 / gather_threads<T, SMEM, FULL>() : 4;
+}
 
 template <typename T, bool CHI2, bool SMEM, bool EDGE, int K, bool MULTI = false, bool FULL = false>
-__global__ void __launch_bounds__(gather_threads<SMEM, FULL>(), gather_min_blocks<SMEM, FULL>())
+__global__ void __launch_bounds__(gather_threads<T, SMEM, FULL>(), gather_min_blocks<T, SMEM, FULL>())
 gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes,
               const __grid_constant__ MultiArg<T, MULTI> multi) {
   using C = cplx_t<T>;
@@ -1871,10 +1875,10 @@ template <typename T> int Launch<T>::gather_blocks_per_sm(bool chi2, size_t wind
   if (window_smem) {
     if (chi2)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gather_kernel<T, true, true, true, 1>,
-                                                    gather_threads<true>(), window_smem);
+                                                    gather_threads<T, true>(), window_smem);
     else
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gather_kernel<T, false, true, true, 1>,
-                                                    gather_threads<true>(), window_smem);
+                                                    gather_threads<T, true>(), window_smem);
   } else {
     if (chi2)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gather_kernel<T, true, false, true, 1>, 256, 0);
@@ -2011,7 +2015,7 @@ cudaError_t Launch<T>::gather(const void* Gw, const GatherParams& gp, const doub
   const GatherT<T> p = GatherT<T>::make(gp);
   const C* g = static_cast<const C*>(Gw);
   const int nodes = (int)(window_smem / sizeof(C));
-  const int threads = window_smem ? gather_threads<true>() : gather_threads<false>();
+  const int threads = window_smem ? gather_threads<T, true>() : gather_threads<T, false>();
   int grid = blocks;
   if (!chi2) {
     int64_t need = (M + threads - 1) / threads;

@@ -305,21 +305,21 @@ template <typename T> int Plane<T>::gather_blocks_per_sm(bool chi2, size_t windo
     if (chi2) {
       constexpr auto kern = gather_kernel<T, true, true, true, 1, false, true>;
       if (ensure_smem_attr<kern>(window_smem) == cudaSuccess)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, gather_threads<true, true>(),
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, gather_threads<T, true, true>(),
                                                       window_smem);
     } else {
       constexpr auto kern = gather_kernel<T, false, true, true, 1, false, true>;
       if (ensure_smem_attr<kern>(window_smem) == cudaSuccess)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, gather_threads<true, true>(),
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, gather_threads<T, true, true>(),
                                                       window_smem);
     }
   } else {
     if (chi2)
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &n, gather_kernel<T, true, false, true, 1, false, true>, gather_threads<false>(), 0);
+          &n, gather_kernel<T, true, false, true, 1, false, true>, gather_threads<T, false>(), 0);
     else
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &n, gather_kernel<T, false, false, true, 1, false, true>, gather_threads<false>(), 0);
+          &n, gather_kernel<T, false, false, true, 1, false, true>, gather_threads<T, false>(), 0);
   }
   (void)cudaGetLastError();
   return n < 1 ? 1 : n;
@@ -336,7 +336,7 @@ cudaError_t Plane<T>::gather(const void* Gw, const GatherParams& gp, const doubl
   int vec = al16(u) && al16(v);
   if (chi2) vec = vec && al16(re) && al16(im) && al16(w);
   const int nodes = (int)(window_smem / sizeof(C));
-  const int threads = window_smem ? gather_threads<true, true>() : gather_threads<false, true>();
+  const int threads = window_smem ? gather_threads<T, true, true>() : gather_threads<T, false, true>();
   int grid = blocks;
   if (!chi2) {
     int64_t need = (M + threads - 1) / threads;
