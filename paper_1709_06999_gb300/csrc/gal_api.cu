@@ -17,6 +17,7 @@
 
 #include "../../include/galario_gb300.h"
 #include "gal_common.cuh"
+#include "gal_fft3.cuh"
 #include "gal_internal.h"
 #include "gal_reorder.h"
 
@@ -150,11 +151,9 @@ cudaError_t grow(gal_ctx* ctx, void** p, size_t* have, size_t need) {
 
 template <typename T> constexpr int prec_index() { return sizeof(T) == 8 ? 1 : 0; }
 
-// the float table holds nxy complex values, the double one nxy more factors
-// of 16 bytes after them
-constexpr size_t twiddle_bytes(int nxy, bool f64) { return (size_t)nxy * (f64 ? 32 : 8); }
-template <typename T> constexpr size_t twiddle_bytes(int nxy) {
-  return twiddle_bytes(nxy, sizeof(T) == 8);
+// a side's twiddle buffer (gal::TwTab)
+constexpr size_t twiddle_bytes(int nxy, bool f64) {
+  return (size_t)gal::kTwUnits * nxy * (f64 ? 16 : 8);
 }
 constexpr int kSinCosLen = 1024;
 
@@ -163,7 +162,7 @@ constexpr int kSinCosLen = 1024;
 template <typename T> int ensure_twiddles(gal_ctx* ctx, int nxy) {
   void*& tw = ctx->tw[prec_index<T>()][log2i(nxy)];
   if (!tw) {
-    GAL_CUDA(ctx, cudaMalloc(&tw, twiddle_bytes<T>(nxy)));
+    GAL_CUDA(ctx, cudaMalloc(&tw, twiddle_bytes(nxy, sizeof(T) == 8)));
     ++g_ws_generation;
     GAL_CUDA(ctx, gal::Launch<T>::twiddles(tw, nxy, 0));
     GAL_CUDA(ctx, cudaStreamSynchronize(0));
@@ -260,7 +259,7 @@ gal::GatherParams gather_params(const gal_ctx* ctx, int nxy, double dxy, double 
   g.phy = dDec;
   g.N = nxy;
   const char* t = static_cast<const char*>(ctx->tw[1][log2i(kSinCosLen)]);  // null until a double call
-  g.sincos = t ? t + 16 * kSinCosLen : nullptr;
+  g.sincos = t ? t + 16 * gal::TwTab<double, 8>::fx(kSinCosLen) : nullptr;
   return g;
 }
 

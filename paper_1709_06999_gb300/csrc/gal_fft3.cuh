@@ -17,6 +17,12 @@
 // (float2) or quarter-warp (double2), and since L is a compile-time constant
 // the padded addresses reduce to a per-thread base plus immediate offsets.
 //
+// Twiddles come staged (TwTab): stage s holds value r of k at V^s - V + (r - 1)
+// Ns + k, so that the lanes of a warp, which hold consecutive k, read
+// consecutive values.  In the plain table W^k they are r L/(Ns R) entries
+// apart, up to a line each, and those reads took most of the L1 cycles of the
+// last stage (column pass of 32 x 465 columns of 1024: 90 us, see col_fft3_kernel).
+//
 // The last stage is run by the caller: last_full() computes it completely,
 // pruned_pair3() evaluates only X[j] and X[L-j] from its input.
 #pragma once
@@ -39,6 +45,37 @@ template <int L, int V> struct P3 {
   static constexpr int padded = L + (L >> lv);
 };
 
+// Layout of a side's twiddle buffer.  The N factors W_N^k come first; then the
+// staged tables of the transforms of length N (column pass, full-plane rows)
+// and N/2 (row pass), L - V entries each.  float: at radix 16 and at radix 8.
+// double: one table of doubles (full-plane rows), then the factors and both
+// tables again in digits for the integer passes (gal_fx.cuh).
+constexpr int kTwUnits = 5;  // a buffer holds kTwUnits N entries
+template <typename T, int V> struct TwTab {
+  static_assert(sizeof(T) == 4 ? (V == 16 || V == 8) : V == 8, "radix");
+  static constexpr bool f64 = sizeof(T) == 8;
+  static __host__ __device__ constexpr size_t col(int N) {
+    return f64 || V == 16 ? (size_t)N : (size_t)5 * N / 2;
+  }
+  static __host__ __device__ constexpr size_t row(int N) {  // float
+    return V == 16 ? (size_t)2 * N : (size_t)7 * N / 2;
+  }
+  static __host__ __device__ constexpr size_t fx(int N) { return (size_t)2 * N; }  // double
+  static __host__ __device__ constexpr size_t fx_col(int N) { return (size_t)3 * N; }
+  static __host__ __device__ constexpr size_t fx_row(int N) { return (size_t)4 * N; }
+};
+// entry i of the staged table of length L at radix V: its exponent in units of 1/L turns
+__host__ __device__ inline int tw_stage_exponent(int L, int V, int i) {
+  int Ns = V, R = V;  // span and radix of the stage
+  for (;;) {
+    if (Ns * V >= L) R = L / Ns;
+    if (i < (R - 1) * Ns) break;
+    i -= (R - 1) * Ns;
+    Ns *= V;
+  }
+  return (i / Ns + 1) * (i % Ns) * (L / (Ns * R));
+}
+
 template <int V> __device__ __forceinline__ int pad3(int a) { return a + (a >> ilog2c(V)); }
 
 // address of element `base + r * step` when step is a multiple of V and base
@@ -50,9 +87,9 @@ template <int V> __device__ __forceinline__ constexpr int pad_step(int step) {
 template <int R, typename C> __device__ __forceinline__ void bfly_any(C* a) { bflyR<R>(a); }
 
 // ---------------------------------------------------------------------------
-// stages 0 .. nstage-2 (all radix V); ST is the stage index
+// stages 0 .. nstage-2 (all radix V); ST is the stage index; tw: staged table
 // ---------------------------------------------------------------------------
-template <int L, int V, int TWS, int ST> struct Head3 {
+template <int L, int V, int ST> struct Head3 {
   using P = P3<L, V>;
   template <typename C, typename Sync>
   static __device__ __forceinline__ void run(C (&v)[V], C* A, C* B, int t, const C* __restrict__ tw,
@@ -76,9 +113,8 @@ template <int L, int V, int TWS, int ST> struct Head3 {
 #pragma unroll
           for (int r = 1; r < V; ++r) v[r] = cmul(v[r], tw1[r - 1]);
         } else {
-          constexpr int F = (L / (Ns * V)) * TWS;
 #pragma unroll
-          for (int r = 1; r < V; ++r) v[r] = cmul(v[r], __ldg(tw + r * F * k));
+          for (int r = 1; r < V; ++r) v[r] = cmul(v[r], __ldg(tw + (Ns - V) + (r - 1) * Ns + k));
         }
       }
       bflyR<V>(v);
@@ -93,21 +129,19 @@ template <int L, int V, int TWS, int ST> struct Head3 {
         for (int r = 0; r < V; ++r) out[base + r * pad_step<V>(Ns)] = v[bfly_out<V>(r)];
       }
       sync();
-      Head3<L, V, TWS, ST + 1>::run(v, A, B, t, tw, tw1, sync);
+      Head3<L, V, ST + 1>::run(v, A, B, t, tw, tw1, sync);
     }
   }
 };
 
 // twiddles of stage 1 for thread t (loop-invariant across sequences)
-template <int L, int V, int TWS, typename C>
+template <int L, int V, typename C>
 __device__ __forceinline__ void load_tw1(C (&tw1)[V - 1], int t, const C* __restrict__ tw) {
   using P = P3<L, V>;
   if constexpr (P::nstage >= 3) {
-    constexpr int Ns = V;
-    constexpr int F = (L / (Ns * V)) * TWS;
-    const int k = t & (Ns - 1);
+    const int k = t & (V - 1);
 #pragma unroll
-    for (int r = 1; r < V; ++r) tw1[r - 1] = __ldg(tw + r * F * k);
+    for (int r = 1; r < V; ++r) tw1[r - 1] = __ldg(tw + (r - 1) * V + k);
   }
 }
 
@@ -118,7 +152,7 @@ template <int L, int V, typename C> __device__ __forceinline__ C* last_input(C* 
 
 // Full last stage (radix R = rlast, span Nsl): v[q R + r] <- X[t + q T + r L/R].
 // Reads `in`; for nstage == 1 the inputs are taken from registers instead.
-template <int L, int V, int TWS, typename C>
+template <int L, int V, typename C>
 __device__ __forceinline__ void last_full(C (&v)[V], const C* in, int t, const C* __restrict__ tw) {
   using P = P3<L, V>;
   constexpr int R = P::rlast, T = P::T;
@@ -136,7 +170,8 @@ __device__ __forceinline__ void last_full(C (&v)[V], const C* in, int t, const C
 #pragma unroll
       for (int r = 0; r < R; ++r) v[q * R + r] = in[pad3<V>(b + r * (L / R))];
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], __ldg(tw + r * b * TWS));
+      for (int r = 1; r < R; ++r)
+        v[q * R + r] = cmul(v[q * R + r], __ldg(tw + (P::Nsl - V) + (r - 1) * P::Nsl + b));
       bflyR<R>(&v[q * R]);
       C o[R];
 #pragma unroll
@@ -158,12 +193,12 @@ __device__ __forceinline__ void store_full(const C (&v)[V], C* out, int t) {
     for (int r = 0; r < R; ++r) out[pad3<V>(t + q * T + r * (L / R))] = v[q * R + r];
 }
 
-// twiddles for pruned_pair at index j (loop-invariant when j is fixed)
-template <int L, int V, int TWS, typename C>
+// twiddles for pruned_pair at index j < Nsl (loop-invariant when j is fixed)
+template <int L, int V, typename C>
 __device__ __forceinline__ void load_twp(C (&twp)[V], int j, const C* __restrict__ tw) {
-  constexpr int R = P3<L, V>::rlast;
+  using P = P3<L, V>;
 #pragma unroll
-  for (int r = 1; r < R; ++r) twp[r - 1] = __ldg(tw + r * j * TWS);
+  for (int r = 1; r < P::rlast; ++r) twp[r - 1] = __ldg(tw + (P::Nsl - V) + (r - 1) * P::Nsl + j);
 }
 
 // X[j] and X[L-j] (X[L] = X[0]) from the last stage's input, 0 <= j < Nsl:

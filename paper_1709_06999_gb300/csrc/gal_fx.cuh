@@ -158,29 +158,17 @@ __device__ __forceinline__ double fx_to(long long v, int q) {
 __device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
 
 // ---------------------------------------------------------------------------
-// The transform: the Stockham plan of gal_fft3.cuh at radix 8.  The factors of
-// the stages between the first and the last are staged in shared memory in the
-// order the lanes read them (stage s: factor r of k at 8^s - 8 + (r - 1) 8^s +
-// k), because from the global table each lane would touch its own line.
+// The transform: the Stockham plan of gal_fft3.cuh at radix 8, with its staged
+// factors in digits.  Those of the stages between the first and the last are
+// kept in shared memory (the first 8^(nstage-1) - 8 entries of the table).
 // ---------------------------------------------------------------------------
 template <int L> struct FxPlan {
   using P = P3<L, 8>;
   static constexpr int ntab = P::nstage >= 3 ? ipowc(8, P::nstage - 1) - 8 : 0;
 };
 
-// fills tab (ntab entries); tw: factors W_{TWS L}^k
-template <int L, int TWS>
-__device__ __forceinline__ void fx_fill_tab(fxtw* tab, const fxtw* __restrict__ tw) {
-  constexpr int n = FxPlan<L>::ntab;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    int Ns = 8, o = i;
-    while (o >= 7 * Ns) {
-      o -= 7 * Ns;
-      Ns *= 8;
-    }
-    const int r = o / Ns + 1, k = o & (Ns - 1);
-    tab[i] = ldg_tw(tw + r * k * (L / (Ns * 8)) * TWS);
-  }
+template <int L> __device__ __forceinline__ void fx_fill_tab(fxtw* tab, const fxtw* __restrict__ tws) {
+  for (int i = threadIdx.x; i < FxPlan<L>::ntab; i += blockDim.x) tab[i] = ldg_tw(tws + i);
 }
 
 template <int L, int ST> struct FxHead {
@@ -209,9 +197,9 @@ template <int L, int ST> struct FxHead {
 };
 
 // last stage, complete: v[q R + r] <- X[t + q T + r L / R]
-template <int L, int TWS>
+template <int L>
 __device__ __forceinline__ void fx_last_full(fx2 (&v)[8], const fx2* in, int t,
-                                             const fxtw* __restrict__ tw) {
+                                             const fxtw* __restrict__ tws) {
   using P = P3<L, 8>;
   constexpr int R = P::rlast, T = P::T;
   if constexpr (P::nstage == 1) {
@@ -223,15 +211,16 @@ __device__ __forceinline__ void fx_last_full(fx2 (&v)[8], const fx2* in, int t,
 #pragma unroll
       for (int r = 0; r < R; ++r) v[q * R + r] = in[pad3<8>(b + r * (L / R))];
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], ldg_tw(tw + r * b * TWS));
+      for (int r = 1; r < R; ++r) 
+        v[q * R + r] = cmul(v[q * R + r], ldg_tw(tws + (P::Nsl - 8) + (r - 1) * P::Nsl + b));
       bflyR<R>(&v[q * R]);
     }
   }
 }
 
 // X[j] and X[L - j] only (pruned_pair3)
-template <int L, int TWS>
-__device__ __forceinline__ void fx_pruned_pair(const fx2* in, int j, const fxtw* __restrict__ tw,
+template <int L>
+__device__ __forceinline__ void fx_pruned_pair(const fx2* in, int j, const fxtw* __restrict__ tws,
                                                fx2& xj, fx2& xmj) {
   using P = P3<L, 8>;
   constexpr int R = P::rlast, Ns = P::Nsl;
@@ -240,7 +229,7 @@ __device__ __forceinline__ void fx_pruned_pair(const fx2* in, int j, const fxtw*
   fx2 a = in[ba], b = in[bb + pad_step<8>(Ns)];
 #pragma unroll
   for (int r = 1; r < R; ++r) {
-    const fxtw w = ldg_tw(tw + r * j * TWS);
+    const fxtw w = ldg_tw(tws + (Ns - 8) + (r - 1) * Ns + j);
     a = cadd(a, cmul(in[ba + r * pad_step<8>(Ns)], w));
     b = cadd(b, cmul(in[bb + (r + 1) * pad_step<8>(Ns)], cconj(w)));
   }

@@ -22,10 +22,7 @@ namespace gal {
 template <int LG> struct FxRowShape {
   static constexpr int M = 1 << LG, N = 2 * M;
   using SH = Shape3<double, M, N, 128, 8>;
-  static constexpr int G = SH::G;
-  // row stride of the work buffers: half a bank row off, so that two rows read
-  // side by side do not collide
-  static constexpr int RS = SH::RS + (G > 1 ? 4 : 0);
+  static constexpr int G = SH::G, RS = SH::RS;
   static constexpr int ntab = FxPlan<M>::ntab;
   // header (barrier, reduction scratch, row scales), factor table, two work
   // buffers, the image rows as they arrive
@@ -54,7 +51,8 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
   const double* __restrict__ image = jb.image;
   const double* __restrict__ beam = BEAM ? jb.beam : nullptr;
   double2* __restrict__ F1 = jb.F1;
-  const fxtw* __restrict__ tw = reinterpret_cast<const fxtw*>(twd + N);
+  const fxtw* __restrict__ tw = reinterpret_cast<const fxtw*>(twd + TwTab<double, 8>::fx(N));
+  const fxtw* __restrict__ tws = reinterpret_cast<const fxtw*>(twd + TwTab<double, 8>::fx_row(N));
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   unsigned* red_max = reinterpret_cast<unsigned*>(smem_raw + 32);   // one per warp, <= 16
@@ -85,7 +83,7 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
       issue(blockIdx.x);
     }
   }
-  fx_fill_tab<M, 2>(tab, tw);
+  fx_fill_tab<M>(tab, tws);
   const Bounds bd = block_bounds(jb.rho2, jb.S, N);  // synchronises
   const bool pruned = P::nstage >= 2 && bd.Kc <= P::Nsl;
   if constexpr (BEAM) grid_dep_wait();  // the beam tables
@@ -131,7 +129,7 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
     FxHead<M, 0>::run(v, A, B, t, tab);
     fx2* in = last_input<M, 8>(A, B);
     if (!pruned) {
-      fx_last_full<M, 2>(v, in, t, tw);
+      fx_last_full<M>(v, in, t, tws);
       in = in == A ? B : A;
       store_full<M, 8>(v, in, t);
       __syncthreads();
@@ -145,7 +143,7 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
       const fx2* x = in0 + gg * RS;
       fx2 zk, zmk;
       if (pruned) {
-        fx_pruned_pair<M, 2>(x, k, tw, zk, zmk);
+        fx_pruned_pair<M>(x, k, tws, zk, zmk);
       } else {
         zk = x[pad3<8>(k & (M - 1))];
         zmk = x[pad3<8>((M - k) & (M - 1))];
@@ -179,7 +177,7 @@ col_fx_kernel(const __grid_constant__ Jobs<ColJob<double>, K> jobs, const double
   const ColJob<double>& jb = jobs.j[K == 1 ? 0 : blockIdx.y];
   const double2* __restrict__ F1 = jb.F1;
   double2* __restrict__ Gw = jb.Gw;
-  const fxtw* __restrict__ tw = reinterpret_cast<const fxtw*>(twd + N);
+  const fxtw* __restrict__ tws = reinterpret_cast<const fxtw*>(twd + TwTab<double, 8>::fx_col(N));
   grid_dep_launch();  // the gather may start its prologue on the SMs we leave idle
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned* red_max = reinterpret_cast<unsigned*>(smem_raw);
@@ -189,7 +187,7 @@ col_fx_kernel(const __grid_constant__ Jobs<ColJob<double>, K> jobs, const double
   fx2* base = reinterpret_cast<fx2*>(smem_raw + S::kHead + (size_t)S::ntab * sizeof(fxtw));
   static_assert(G <= 256 && SH::threads <= 512, "header");
   const int g = threadIdx.x / TT, t = threadIdx.x - g * TT;
-  fx_fill_tab<N, 1>(tab, tw);
+  fx_fill_tab<N>(tab, tws);
   const Bounds bd = block_bounds(jb.rho2, jb.S, N);  // synchronises
   const int ncol = jb.full ? full_cols(bd, N).W : bd.Kc;
   const int kmax = N / 2 - bd.r0;
@@ -213,14 +211,14 @@ col_fx_kernel(const __grid_constant__ Jobs<ColJob<double>, K> jobs, const double
     if (pruned) {
       for (int j = t; j <= kmax; j += TT) {
         fx2 xj, xmj;
-        fx_pruned_pair<N, 1>(in, j, tw, xj, xmj);
+        fx_pruned_pair<N>(in, j, tws, xj, xmj);
         if (act) {
           Gw[(size_t)(kmax + j) * ncol + c] = value(xj, sc.q, sc.bad);
           if (j > 0) Gw[(size_t)(kmax - j) * ncol + c] = value(xmj, sc.q, sc.bad);
         }
       }
     } else {
-      fx_last_full<N, 1>(v, in, t, tw);
+      fx_last_full<N>(v, in, t, tws);
       fx2* o = in == A ? B : A;
       store_full<N, 8>(v, o, t);
       if (t == 0) col_q[g] = sc.bad ? INT_MAX : sc.q;

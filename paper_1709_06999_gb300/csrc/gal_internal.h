@@ -53,7 +53,7 @@ template <typename T> struct Launch {
   // takes `edge` = false only when the window is known to be pruned (no uv
   // point can reach the edge of the half spectrum).
   static int gather_blocks_per_sm(bool chi2, size_t window_smem);
-  // tw: 2 N values; in double another N factors of 16 bytes follow (gal_fx.cuh)
+  // tw: kTwUnits N complex values (TwTab)
   static cudaError_t twiddles(void* tw, int N, cudaStream_t st);
   static cudaError_t extent(const T* u, const T* v, int64_t M, double* rho2, int blocks,
                             cudaStream_t st);

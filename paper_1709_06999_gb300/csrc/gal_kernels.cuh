@@ -27,17 +27,43 @@
 namespace gal {
 
 // ---------------------------------------------------------------------------
-// twiddles: tw[k] = exp(-2 pi i k / N), k = 0 .. N-1
+// twiddles: tw[k] = exp(-2 pi i k / N), k = 0 .. N-1, and the staged tables (TwTab)
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void twiddle_kernel(cplx_t<T>* __restrict__ tw, int N) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= N) return;
-  double s, c;
-  sincospi(-2.0 * (double)k / (double)N, &s, &c);
-  tw[k] = mkc((T)c, (T)s);
-  // the double table is followed by the same factors for the integer passes
-  if constexpr (sizeof(T) == 8) reinterpret_cast<fxtw*>(tw + N)[k] = fx_factor(c, s);
+  const int stride = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
+  auto factor = [&](int k) {  // W_N^k
+    double s, c;
+    sincospi(-2.0 * (double)k / (double)N, &s, &c);
+    return make_double2(c, s);
+  };
+  auto put = [&](cplx_t<T>* to, int n, auto&& exponent) {
+    for (int k = t0; k < n; k += stride) {
+      const double2 w = factor(exponent(k));
+      to[k] = mkc((T)w.x, (T)w.y);
+    }
+  };
+  auto col = [&](int V) { return [=](int i) { return tw_stage_exponent(N, V, i); }; };
+  auto row = [&](int V) { return [=](int i) { return 2 * tw_stage_exponent(N / 2, V, i); }; };
+  auto plain = [](int k) { return k; };
+  put(tw, N, plain);
+  if constexpr (sizeof(T) == 4) {
+    put(tw + TwTab<T, 16>::col(N), N - 16, col(16));
+    put(tw + TwTab<T, 16>::row(N), N / 2 - 16, row(16));
+    put(tw + TwTab<T, 8>::col(N), N - 8, col(8));
+    put(tw + TwTab<T, 8>::row(N), N / 2 - 8, row(8));
+  } else {
+    put(tw + TwTab<T, 8>::col(N), N - 8, col(8));
+    auto put_fx = [&](size_t off, int n, auto&& exponent) {
+      for (int k = t0; k < n; k += stride) {
+        const double2 w = factor(exponent(k));
+        reinterpret_cast<fxtw*>(tw + off)[k] = fx_factor(w.x, w.y);
+      }
+    };
+    put_fx(TwTab<T, 8>::fx(N), N, plain);
+    put_fx(TwTab<T, 8>::fx_col(N), N - 8, col(8));
+    put_fx(TwTab<T, 8>::fx_row(N), N / 2 - 8, row(8));
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -369,7 +395,14 @@ template <typename T, int L, int NSEQ, int MINT = 128, int VV = FftV<T>::V> stru
   static constexpr int G0 = P::T >= MINT ? 1 : MINT / P::T;
   static constexpr int G = G0 < NSEQ ? G0 : NSEQ;
   static constexpr int threads = G * P::T;
-  static constexpr int RS = (P::padded * (int)sizeof(C) + 15) / 16 * 16 / (int)sizeof(C);
+  // sequence stride: with several sequences to a block, 1/G of a bank row (at
+  // least 16 bytes) off a whole one, so that values read side by side from the G
+  // sequences (the unpacking of a row group, the rows of a column group) do not
+  // collide: four columns of 1024 at a stride of 0 mod 128 bytes made each of
+  // those reads four times as long
+  static constexpr int RS0 = (P::padded * (int)sizeof(C) + 15) / 16 * 16 / (int)sizeof(C);
+  static constexpr int kOff = (G >= 8 ? 16 : 128 / G) / (int)sizeof(C), kRow = 128 / (int)sizeof(C);
+  static constexpr int RS = G == 1 ? RS0 : RS0 + (kRow + kOff - RS0 % kRow) % kRow;
 };
 
 // Row pass: row i' of F1 (column-major) = first Kc bins of the real-to-complex FFT
@@ -420,20 +453,21 @@ row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>
   C* base = reinterpret_cast<C*>(smem_raw + 128);
   const int g = threadIdx.x / TT, t = threadIdx.x - g * TT;
   const Bounds bd = block_bounds(rho2, S, N);
+  const C* __restrict__ tws = tw + TwTab<T, V>::row(N);
   C tw1[V - 1];
-  load_tw1<M, V, 2>(tw1, t, tw);
+  load_tw1<M, V>(tw1, t, tws);
   const bool pruned = P::nstage >= 2 && bd.Kc <= P::Nsl;
   const bool one_j = bd.Kc <= TT;
   C twp[V];
   C wj = mkc((T)0, (T)0);
   if (pruned && one_j && t < bd.Kc) {
-    load_twp<M, V, 2>(twp, t, tw);
+    load_twp<M, V>(twp, t, tws);
     wj = __ldg(tw + t);
   }
   auto sync = [] { __syncthreads(); };
   // Transform the group held in registers v (stage-0 layout), A, B: buffers.
   auto transform = [&](C (&v)[V], C* A, C* B, int row) {
-    Head3<M, V, 2, 0>::run(v, A, B, t, tw, tw1, sync);
+    Head3<M, V, 0>::run(v, A, B, t, tws, tw1, sync);
     C* in = last_input<M, V>(A, B);
     C* out = F1 + row;  // column-major: bin j of this row at out[j N]
     if (pruned) {
@@ -444,13 +478,13 @@ row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>
           out[(size_t)j * N] = r2c_unpack(zj, zmj, wj);
         } else {
           C tj[V];
-          load_twp<M, V, 2>(tj, j, tw);
+          load_twp<M, V>(tj, j, tws);
           pruned_pair3<M, V>(in, j, tj, zj, zmj);
           out[(size_t)j * N] = r2c_unpack(zj, zmj, __ldg(tw + j));
         }
       }
     } else {
-      last_full<M, V, 2>(v, in, t, tw);
+      last_full<M, V>(v, in, t, tws);
       C* o = in == A ? B : A;
       store_full<M, V>(v, o, t);
       __syncthreads();
@@ -594,6 +628,7 @@ row_fft3_ldg_kernel(const __grid_constant__ Jobs<RowJob<float>, K> jobs, const f
   const float* __restrict__ image = jb.image;
   const float* __restrict__ beam = BEAM ? jb.beam : nullptr;
   C* __restrict__ F1 = jb.F1;
+  const C* __restrict__ tws = tw + TwTab<float, V>::row(N);
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C* A = reinterpret_cast<C*>(smem_raw);
   C* B = A + RS;
@@ -636,11 +671,11 @@ row_fft3_ldg_kernel(const __grid_constant__ Jobs<RowJob<float>, K> jobs, const f
   if (fast) {
     if (t < bd.Kc) wj = __ldg(tw + t);
   } else {
-    load_tw1<M, V, 2>(tw1, t, tw);
+    load_tw1<M, V>(tw1, t, tws);
   }
   C twp[V];
   if (!fast && pruned && t < bd.Kc) {
-    load_twp<M, V, 2>(twp, t, tw);
+    load_twp<M, V>(twp, t, tws);
     wj = __ldg(tw + t);
   }
   auto sync = [] { __syncthreads(); };
@@ -690,7 +725,7 @@ row_fft3_ldg_kernel(const __grid_constant__ Jobs<RowJob<float>, K> jobs, const f
         out[(size_t)t * N] = r2c_unpack(zj, t == 0 ? zj : zhi[t], wj);
       }
     } else {
-      Head3<M, V, 2, 0>::run(v, A, B, t, tw, tw1, sync);
+      Head3<M, V, 0>::run(v, A, B, t, tws, tw1, sync);
       C* in = last_input<M, V>(A, B);
       if (pruned) {
         for (int j = t; j < bd.Kc; j += TT) {
@@ -700,13 +735,13 @@ row_fft3_ldg_kernel(const __grid_constant__ Jobs<RowJob<float>, K> jobs, const f
             out[(size_t)j * N] = r2c_unpack(zj, zmj, wj);
           } else {
             C tj[V];
-            load_twp<M, V, 2>(tj, j, tw);
+            load_twp<M, V>(tj, j, tws);
             pruned_pair3<M, V>(in, j, tj, zj, zmj);
             out[(size_t)j * N] = r2c_unpack(zj, zmj, __ldg(tw + j));
           }
         }
       } else {
-        last_full<M, V, 2>(v, in, t, tw);
+        last_full<M, V>(v, in, t, tws);
         C* o = in == A ? B : A;
         store_full<M, V>(v, o, t);
         __syncthreads();
@@ -751,13 +786,14 @@ col_fft3_kernel(const __grid_constant__ Jobs<ColJob<T>, K> jobs, const cplx_t<T>
   const int g = threadIdx.x / TT, t = threadIdx.x - g * TT;
   const Bounds bd = block_bounds(rho2, S, N);
   const int ncol = jb.full ? full_cols(bd, N).W : bd.Kc;  // window columns (and pitch)
+  const C* __restrict__ tws = tw + TwTab<T, V>::col(N);
   C tw1[V - 1];
-  load_tw1<N, V, 1>(tw1, t, tw);
+  load_tw1<N, V>(tw1, t, tws);
   const int kmax = N / 2 - bd.r0;
   const bool pruned = P::nstage >= 2 && bd.r0 > 0 && kmax < P::Nsl;
   const bool one_j = kmax < TT;
   C twp[V];
-  if (pruned && one_j && t <= kmax) load_twp<N, V, 1>(twp, t, tw);
+  if (pruned && one_j && t <= kmax) load_twp<N, V>(twp, t, tws);
   C* A = base + (size_t)g * RS;
   C* B = base + (size_t)(G + g) * RS;
   auto sync = [] { __syncthreads(); };
@@ -768,7 +804,7 @@ col_fft3_kernel(const __grid_constant__ Jobs<ColJob<T>, K> jobs, const cplx_t<T>
     C v[V];
 #pragma unroll
     for (int r = 0; r < V; ++r) v[r] = act ? F1[(size_t)c * N + t + r * TT] : mkc((T)0, (T)0);
-    Head3<N, V, 1, 0>::run(v, A, B, t, tw, tw1, sync);
+    Head3<N, V, 0>::run(v, A, B, t, tws, tw1, sync);
     C* in = last_input<N, V>(A, B);
     if (pruned) {
       for (int j = t; j <= kmax; j += TT) {
@@ -777,7 +813,7 @@ col_fft3_kernel(const __grid_constant__ Jobs<ColJob<T>, K> jobs, const cplx_t<T>
           pruned_pair3<N, V>(in, j, twp, xj, xmj);
         } else {
           C tj[V];
-          load_twp<N, V, 1>(tj, j, tw);
+          load_twp<N, V>(tj, j, tws);
           pruned_pair3<N, V>(in, j, tj, xj, xmj);
         }
         if (act) {
@@ -786,7 +822,7 @@ col_fft3_kernel(const __grid_constant__ Jobs<ColJob<T>, K> jobs, const cplx_t<T>
         }
       }
     } else {
-      last_full<N, V, 1>(v, in, t, tw);
+      last_full<N, V>(v, in, t, tws);
       C* o = in == A ? B : A;
       store_full<N, V>(v, o, t);
       __syncthreads();

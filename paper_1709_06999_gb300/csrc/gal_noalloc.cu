@@ -16,6 +16,7 @@
 
 #include "../../include/galario_gb300.h"
 #include "gal_common.cuh"
+#include "gal_fft3.cuh"
 #include "gal_internal.h"
 
 namespace {
@@ -25,7 +26,7 @@ constexpr size_t kSpecElems = (size_t)kMaxN * (kMaxN / 2 + 1);     // half spect
 constexpr int kMaxBlocks = 8192;                                  // reduction partials
 constexpr size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 constexpr size_t kOffTw = 0;
-constexpr size_t kOffF1 = kOffTw + align256(sizeof(float2) * kMaxN);
+constexpr size_t kOffF1 = kOffTw + align256(sizeof(float2) * gal::kTwUnits * kMaxN);
 constexpr size_t kOffGw = kOffF1 + align256(sizeof(float2) * kSpecElems);
 constexpr size_t kOffPartials = kOffGw + align256(2 * sizeof(float2) * kSpecElems);
 constexpr size_t kOffRho2 = kOffPartials + align256(sizeof(double) * kMaxBlocks);

@@ -17,7 +17,8 @@ template <typename T> constexpr int plane_max_lg() { return col3_max_lg<T>(); }
 // Length-L complex transform of one row held in registers (v[r] at shifted
 // index t + r T, stage-0 layout), and the store of its kept bins to row
 // `row` of F1: bin k mod L at column k + fc.lo for k = -fc.lo .. fc.hi.
-// Every thread of the block calls it (it synchronises); `act` masks the store.
+// Every thread of the block calls it (it synchronises); `act` masks the store;
+// tw: staged twiddles.
 template <typename T, int L> struct C2CRow {
   using C = cplx_t<T>;
   using P = P3<L, FftV<T>::V>;
@@ -28,7 +29,7 @@ template <typename T, int L> struct C2CRow {
                                              const C (&twp)[V], bool pruned, bool one_j,
                                              int kmax, const FullCols& fc, bool act, int row,
                                              C* __restrict__ F1, Sync&& sync) {
-    Head3<L, V, 1, 0>::run(v, A, B, t, tw, tw1, sync);
+    Head3<L, V, 0>::run(v, A, B, t, tw, tw1, sync);
     C* in = last_input<L, V>(A, B);
     if (pruned) {
       for (int j = t; j <= kmax; j += TT) {
@@ -37,7 +38,7 @@ template <typename T, int L> struct C2CRow {
           pruned_pair3<L, V>(in, j, twp, xj, xmj);
         } else {
           C tj[V];
-          load_twp<L, V, 1>(tj, j, tw);
+          load_twp<L, V>(tj, j, tw);
           pruned_pair3<L, V>(in, j, tj, xj, xmj);
         }
         if (act) {
@@ -46,7 +47,7 @@ template <typename T, int L> struct C2CRow {
         }
       }
     } else {
-      last_full<L, V, 1>(v, in, t, tw);
+      last_full<L, V>(v, in, t, tw);
       C* o = in == A ? B : A;
       store_full<L, V>(v, o, t);
       __syncthreads();
@@ -80,12 +81,13 @@ row_c2c_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>*
   const Bounds bd = block_bounds(jb.rho2, jb.S, N);
   const FullCols fc = full_cols(bd, N);
   const int kmax = fc.lo > fc.hi ? fc.lo : fc.hi;
+  const C* __restrict__ tws = tw + TwTab<T, V>::col(N);  // staged twiddles of length N
   C tw1[V - 1];
-  load_tw1<N, V, 1>(tw1, t, tw);
+  load_tw1<N, V>(tw1, t, tws);
   const bool pruned = P::nstage >= 2 && kmax < P::Nsl;
   const bool one_j = kmax < TT;
   C twp[V];
-  if (pruned && one_j && t <= kmax) load_twp<N, V, 1>(twp, t, tw);
+  if (pruned && one_j && t <= kmax) load_twp<N, V>(twp, t, tws);
   C* A = base + (size_t)g * RS;
   C* B = base + (size_t)(G + g) * RS;
   auto sync = [] { __syncthreads(); };
@@ -111,7 +113,7 @@ row_c2c_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>*
       }
       v[r] = mkc(x, (T)0);
     }
-    C2CRow<T, N>::run(v, A, B, t, tw, tw1, twp, pruned, one_j, kmax, fc, act, row, F1, sync);
+    C2CRow<T, N>::run(v, A, B, t, tws, tw1, twp, pruned, one_j, kmax, fc, act, row, F1, sync);
   }
 }
 
@@ -142,12 +144,13 @@ row_c2c_tma_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs,
   const Bounds bd = block_bounds(jb.rho2, jb.S, N);
   const FullCols fc = full_cols(bd, N);
   const int kmax = fc.lo > fc.hi ? fc.lo : fc.hi;
+  const C* __restrict__ tws = tw + TwTab<T, V>::col(N);  // staged twiddles of length N
   C tw1[V - 1];
-  load_tw1<N, V, 1>(tw1, t, tw);
+  load_tw1<N, V>(tw1, t, tws);
   const bool pruned = P::nstage >= 2 && kmax < P::Nsl;
   const bool one_j = kmax < TT;
   C twp[V];
-  if (pruned && one_j && t <= kmax) load_twp<N, V, 1>(twp, t, tw);
+  if (pruned && one_j && t <= kmax) load_twp<N, V>(twp, t, tws);
   C* A = base + (size_t)g * RS;
   C* B = base + (size_t)(G + g) * RS;
   auto sync = [] { __syncthreads(); };
@@ -207,7 +210,7 @@ row_c2c_tma_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs,
       fence_proxy_async_smem();
       issue(it + 2);
     }
-    C2CRow<T, N>::run(v, A, B, t, tw, tw1, twp, pruned, one_j, kmax, fc, true, row, jb.F1, sync);
+    C2CRow<T, N>::run(v, A, B, t, tws, tw1, twp, pruned, one_j, kmax, fc, true, row, jb.F1, sync);
   }
 }
 
