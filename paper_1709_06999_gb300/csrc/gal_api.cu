@@ -383,7 +383,7 @@ template <typename T> int tune_fft(gal_ctx* ctx, int nxy, cudaStream_t st, int* 
                                       S, ctx->err, nullptr, st, r);
     }, &row[k]));
     GAL_TRY(best_of([&] {
-      return gal::Launch<T>::col_pass(ctx->F1, ctx->Gw, nxy, tw, ctx->rho2, S, 0, false, st, r);
+      return gal::Launch<T>::col_pass(ctx->F1, ctx->Gw, nxy, tw, ctx->rho2, S, 0, false, false, st, r);
     }, &col[k]));
   }
   ctx->event_pool.push_back(a);
@@ -419,10 +419,12 @@ int spectrum(gal_ctx* ctx, const T* image, const T* I, const gal::SweepParams& s
   plan_lookup<T>(ctx->device, nxy, &rv, &cv);
   GAL_TRY(stage(ctx, 1, st, [&] {
     if (full) return gal::Plane<T>::rows(image, I, sp, nxy, tw, ctx->F1, rho2, S, beam, ctx->err, st);
-    return gal::Launch<T>::row_pass(image, I, sp, nxy, tw, ctx->F1, rho2, S, ctx->err, beam, st, rv);
+    return gal::Launch<T>::row_pass(image, I, sp, nxy, tw, ctx->F1, rho2, S, ctx->err, beam, st, rv,
+                                    kc_hint);
   }));
   GAL_TRY(stage(ctx, 2, st, [&] {
-    return gal::Launch<T>::col_pass(ctx->F1, ctx->Gw, nxy, tw, rho2, S, kc_hint, full, st, cv);
+    const bool even = I && !beam && !full && gal::Launch<T>::even_profile(nxy);
+    return gal::Launch<T>::col_pass(ctx->F1, ctx->Gw, nxy, tw, rho2, S, kc_hint, full, even, st, cv);
   }));
   return GAL_OK;
 }

@@ -29,12 +29,12 @@ inline int chunk_of(const BatchShape& sh) {
 // rows: the chunk `idx[0..n)` of items, all of length 2^(LG+1), all swept
 // (SWEEP) or all images, all with a beam (BEAM, its tables already computed
 // earlier in the stream) or none
-template <typename T, int LG, bool SWEEP, bool BEAM, int V = FftV<T>::V>
+template <typename T, int LG, bool SWEEP, bool BEAM, int V = FftV<T>::V, bool PAIRS = false>
 cudaError_t rows(const BatchItem* it, const int* idx, int n, const void* tw, int* err,
                  const BatchShape& sh, cudaStream_t st) {
   using C = cplx_t<T>;
   constexpr int M = 1 << LG, N = 2 * M;
-  using SH = Shape3<T, M, N, 128, V>;
+  using SH = Shape3<T, M, N, row_min_threads(PAIRS), V>;
   Jobs<RowJob<T>, kBatchJobs> jb{};
   for (int k = 0; k < n; ++k) {
     const BatchItem& b = it[idx[k]];
@@ -55,7 +55,7 @@ cudaError_t rows(const BatchItem* it, const int* idx, int n, const void* tw, int
     if (x < 1) return cudaErrorInvalidConfiguration;
     kern<<<dim3(x, n), RowLdgShape::TT, RowLdgShape::smem, st>>>(jb, twc);
   } else if constexpr (!SWEEP) {
-    constexpr auto kern = row_fft3_kernel<T, LG, true, false, kBatchJobs, BEAM, 128, 2, V>;
+    constexpr auto kern = row_fft3_kernel<T, LG, true, false, kBatchJobs, BEAM, row_min_threads(PAIRS), 2, V>;
     const size_t smem = 128 + (size_t)3 * SH::G * SH::RS * sizeof(C);
     cudaError_t e = ensure_smem_attr<kern>(smem);
     if (e) return e;
@@ -70,11 +70,12 @@ cudaError_t rows(const BatchItem* it, const int* idx, int n, const void* tw, int
     if (x < 1) x = 1;
     kern<<<dim3(x, n), SH::threads, smem, st>>>(jb, twc, err);
   } else {
-    constexpr auto kern = row_fft3_kernel<T, LG, false, true, kBatchJobs, BEAM, 128, 2, V>;
+    constexpr auto kern = row_fft3_kernel<T, LG, false, true, kBatchJobs, BEAM, row_min_threads(PAIRS), 2, V>;
     const size_t smem = 128 + (size_t)2 * SH::G * SH::RS * sizeof(C);
     const cudaError_t e = ensure_smem_attr<kern>(smem);
     if (e) return e;
-    kern<<<dim3(N / SH::G, n), SH::threads, smem, st>>>(jb, twc, err);
+    const int groups = ((even_rows<T, SWEEP, BEAM>(N) ? M + 1 : N) + SH::G - 1) / SH::G;
+    kern<<<dim3(groups, n), SH::threads, smem, st>>>(jb, twc, err);
   }
   return cudaGetLastError();
 }
@@ -106,7 +107,7 @@ cudaError_t cols(const BatchItem* it, const int* idx, int n, const void* tw, cud
   for (int k = 0; k < n; ++k) {
     const BatchItem& b = it[idx[k]];
     jb.j[k] = ColJob<T>{static_cast<const C*>(b.F1), static_cast<C*>(b.Gw), b.rho2, b.S,
-                        b.full ? 1 : 0};
+                        b.full ? 1 : 0, b.I && !b.beam && !b.full && even_rows<T, true, false>(N) ? 1 : 0};
     kc = b.ncol > kc ? b.ncol : kc;
   }
   if constexpr (sizeof(T) == 8) {
@@ -253,6 +254,11 @@ cudaError_t BatchLaunch<T>::rows(const BatchItem* it, int n, const void* const* 
       } else {
         auto go = [&](auto v_c) {
           constexpr int VV = decltype(v_c)::value;
+          if constexpr (row_pairs_exist<T, LG, false>()) {
+            if (b0.Kc > kRowPairsKc && !b0.I)
+              return b0.beam ? batch::rows<T, LG, false, true, VV, true>(it, idx, m, tw[lg], err, sh, st)
+                             : batch::rows<T, LG, false, false, VV, true>(it, idx, m, tw[lg], err, sh, st);
+          }
           if (b0.beam)
             return b0.I ? batch::rows<T, LG, true, true, VV>(it, idx, m, tw[lg], err, sh, st)
                         : batch::rows<T, LG, false, true, VV>(it, idx, m, tw[lg], err, sh, st);

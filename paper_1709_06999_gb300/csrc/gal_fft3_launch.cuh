@@ -26,9 +26,22 @@ template <auto Kern> int row_ldg_grid(int n) {
   return x > RowLdgShape::N ? RowLdgShape::N : x;
 }
 
+// Least threads to a block of row_fft3_kernel: 128.  Rows of 8192 pixels (256
+// threads) whose window is wider than the pruned last stage come in pairs, so
+// that the stores of a column of F1, 8 bytes a row, fill half a sector instead
+// of a quarter (the whole call with a beam, 1642 columns kept: 419 -> 389 us);
+// with narrow windows a row to a block is faster (123 columns: 88 against 91 us).
+// Rows of 2048 in fours: 1 % faster with 413 columns kept, 3 % slower in batches
+// with 40, so they stay in pairs.
+constexpr int row_min_threads(bool pairs) { return pairs ? 512 : 128; }
+template <typename T, int LG, bool SWEEP> constexpr bool row_pairs_exist() {
+  return sizeof(T) == 4 && LG == 12 && !SWEEP;
+}
+constexpr int kRowPairsKc = 256;  // spans of the pruned last stage of 4096 points
+
 // A row pass with a beam follows beam_table_kernel in the stream and is
 // launched as its programmatic dependent (BEAM kernels wait for the tables).
-template <typename T, int LG, bool SWEEP, bool BEAM, int V = FftV<T>::V>
+template <typename T, int LG, bool SWEEP, bool BEAM, int V = FftV<T>::V, bool PAIRS = false>
 cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc, int* err,
                              cudaStream_t st) {
   using C = cplx_t<T>;
@@ -46,12 +59,12 @@ cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc,
     kern<<<grid, RowLdgShape::TT, RowLdgShape::smem, st>>>(jb, twc);
     return cudaGetLastError();
   } else {
-    using SH = Shape3<T, M, N, 128, V>;
-    constexpr auto kern = row_fft3_kernel<T, LG, !SWEEP, SWEEP, 1, BEAM, 128, 2, V>;
+    using SH = Shape3<T, M, N, row_min_threads(PAIRS), V>;
+    constexpr auto kern = row_fft3_kernel<T, LG, !SWEEP, SWEEP, 1, BEAM, row_min_threads(PAIRS), 2, V>;
     const size_t smem = 128 + (size_t)(SWEEP ? 2 : 3) * SH::G * SH::RS * sizeof(C);
     cudaError_t e = ensure_smem_attr<kern>(smem);
     if (e) return e;
-    int grid = N / SH::G;
+    int grid = ((even_rows<T, SWEEP, BEAM>(N) ? M + 1 : N) + SH::G - 1) / SH::G;
     if constexpr (!SWEEP) {  // persistent blocks over the TMA row ring
       int per_sm = 0;
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SH::threads, smem);
@@ -74,7 +87,7 @@ template <typename T, int N> constexpr bool has_alt_radix() {
 template <typename T, int LG, bool SWEEP>
 cudaError_t launch_row3(const T* image, const T* I, const SweepParams& sp, const void* tw,
                         void* F1, const double* rho2, double S, int* err, const T* beam,
-                        cudaStream_t st, int radix) {
+                        cudaStream_t st, int radix, int kc) {
   using C = cplx_t<T>;
   const C* twc = static_cast<const C*>(tw);
   Jobs<RowJob<T>, 1> jb;
@@ -86,19 +99,26 @@ cudaError_t launch_row3(const T* image, const T* I, const SweepParams& sp, const
       return launch_row3_kern<T, LG, SWEEP, false, kAltRadix>(jb, twc, err, st);
     }
   }
+  if constexpr (row_pairs_exist<T, LG, SWEEP>()) {
+    if (kc > kRowPairsKc) {
+      if (beam) return launch_row3_kern<T, LG, SWEEP, true, FftV<T>::V, true>(jb, twc, err, st);
+      return launch_row3_kern<T, LG, SWEEP, false, FftV<T>::V, true>(jb, twc, err, st);
+    }
+  }
   if (beam) return launch_row3_kern<T, LG, SWEEP, true>(jb, twc, err, st);
   return launch_row3_kern<T, LG, SWEEP, false>(jb, twc, err, st);
 }
 
 template <typename T, int LG, int V = FftV<T>::V>
 cudaError_t launch_col3_kern(const void* F1, void* Gw, const void* tw, const double* rho2, double S,
-                             int kc_hint, bool full, cudaStream_t st) {
+                             int kc_hint, bool full, bool even, cudaStream_t st) {
   using C = cplx_t<T>;
   constexpr int N = 1 << LG;
   const int P = full ? N : N / 2 + 1;  // most window columns
   const int kc = kc_hint > 0 && kc_hint <= P ? kc_hint : P;
   Jobs<ColJob<T>, 1> jb;
-  jb.j[0] = ColJob<T>{static_cast<const C*>(F1), static_cast<C*>(Gw), rho2, S, full ? 1 : 0};
+  jb.j[0] = ColJob<T>{static_cast<const C*>(F1), static_cast<C*>(Gw), rho2, S, full ? 1 : 0,
+                      even ? 1 : 0};
   if constexpr (sizeof(T) == 8) {  // double columns: on integers
     return launch_col_fx<LG, 1>(jb, 1, kc, true, static_cast<const C*>(tw), st);
   } else {
@@ -117,41 +137,41 @@ cudaError_t launch_col3_kern(const void* F1, void* Gw, const void* tw, const dou
 
 template <typename T, int LG>
 cudaError_t launch_col3(const void* F1, void* Gw, const void* tw, const double* rho2, double S,
-                        int kc_hint, bool full, cudaStream_t st, int radix) {
+                        int kc_hint, bool full, bool even, cudaStream_t st, int radix) {
   if constexpr (has_alt_radix<T, (1 << LG)>()) {
     if (radix == kAltRadix)
-      return launch_col3_kern<T, LG, kAltRadix>(F1, Gw, tw, rho2, S, kc_hint, full, st);
+      return launch_col3_kern<T, LG, kAltRadix>(F1, Gw, tw, rho2, S, kc_hint, full, even, st);
   }
-  return launch_col3_kern<T, LG>(F1, Gw, tw, rho2, S, kc_hint, full, st);
+  return launch_col3_kern<T, LG>(F1, Gw, tw, rho2, S, kc_hint, full, even, st);
 }
 
 template <typename T, int LG>
 cudaError_t row3_switch(int lg, const T* image, const T* I, const SweepParams& sp,
                         const void* tw, void* F1, const double* rho2, double S, int* err,
-                        const T* beam, cudaStream_t st, int radix) {
+                        const T* beam, cudaStream_t st, int radix, int kc) {
   if constexpr (LG > 12) {
     return cudaErrorNotSupported;
   } else {
     if (lg == LG) {
-      if (I) return launch_row3<T, LG, true>(image, I, sp, tw, F1, rho2, S, err, beam, st, radix);
-      return launch_row3<T, LG, false>(image, I, sp, tw, F1, rho2, S, err, beam, st, radix);
+      if (I) return launch_row3<T, LG, true>(image, I, sp, tw, F1, rho2, S, err, beam, st, radix, kc);
+      return launch_row3<T, LG, false>(image, I, sp, tw, F1, rho2, S, err, beam, st, radix, kc);
     }
-    return row3_switch<T, LG + 1>(lg, image, I, sp, tw, F1, rho2, S, err, beam, st, radix);
+    return row3_switch<T, LG + 1>(lg, image, I, sp, tw, F1, rho2, S, err, beam, st, radix, kc);
   }
 }
 
 // largest column length with both ping-pong buffers in shared memory:
 // 8192 float2 (2 x 8704 x 8 B) but 4096 double2 (8192 would need 295 KB)
-template <typename T> constexpr int col3_max_lg() { return sizeof(T) == 4 ? 13 : 12; }
+template <typename T> constexpr int col3_max_lg() { return max_col_lg<T>(); }
 
 template <typename T, int LG>
 cudaError_t col3_switch(int lg, const void* F1, void* Gw, const void* tw, const double* rho2,
-                        double S, int kc_hint, bool full, cudaStream_t st, int radix) {
+                        double S, int kc_hint, bool full, bool even, cudaStream_t st, int radix) {
   if constexpr (LG > col3_max_lg<T>()) {
     return cudaErrorNotSupported;
   } else {
-    if (lg == LG) return launch_col3<T, LG>(F1, Gw, tw, rho2, S, kc_hint, full, st, radix);
-    return col3_switch<T, LG + 1>(lg, F1, Gw, tw, rho2, S, kc_hint, full, st, radix);
+    if (lg == LG) return launch_col3<T, LG>(F1, Gw, tw, rho2, S, kc_hint, full, even, st, radix);
+    return col3_switch<T, LG + 1>(lg, F1, Gw, tw, rho2, S, kc_hint, full, even, st, radix);
   }
 }
 
@@ -164,16 +184,16 @@ inline int ilog2i(int n) {
 template <typename T>
 cudaError_t row_fft3(const T* image, const T* I, const SweepParams& sp, int N, const void* tw,
                      void* F1, const double* rho2, double S, int* err, const T* beam,
-                     cudaStream_t st, int radix) {
+                     cudaStream_t st, int radix, int kc) {
   constexpr int LG0 = ilog2c(FftV<T>::V);
-  return row3_switch<T, LG0>(ilog2i(N / 2), image, I, sp, tw, F1, rho2, S, err, beam, st, radix);
+  return row3_switch<T, LG0>(ilog2i(N / 2), image, I, sp, tw, F1, rho2, S, err, beam, st, radix, kc);
 }
 
 template <typename T>
 cudaError_t col_fft3(const void* F1, void* Gw, int N, const void* tw, const double* rho2, double S,
-                     int kc_hint, bool full, cudaStream_t st, int radix) {
+                     int kc_hint, bool full, bool even, cudaStream_t st, int radix) {
   constexpr int LG0 = ilog2c(FftV<T>::V);
-  return col3_switch<T, LG0>(ilog2i(N), F1, Gw, tw, rho2, S, kc_hint, full, st, radix);
+  return col3_switch<T, LG0>(ilog2i(N), F1, Gw, tw, rho2, S, kc_hint, full, even, st, radix);
 }
 
 }  // namespace gal

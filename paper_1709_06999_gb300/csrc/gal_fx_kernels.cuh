@@ -64,7 +64,9 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
   double* slot = reinterpret_cast<double*>(B0 + G * RS);
   static_assert(G <= 64 && SH::threads <= 512, "header");
   const int g = threadIdx.x / TT, t = threadIdx.x - g * TT;
-  const int ngroups = N / G;
+  constexpr bool EVEN = even_rows<double, SWEEP, BEAM>(N);  // rows 0 .. N/2 only
+  constexpr int LD = EVEN ? kEvenRows(N) : N;
+  constexpr int ngroups = EVEN ? (M + 1 + G - 1) / G : N / G;
   const uint32_t half_bytes = (uint32_t)(M * sizeof(double));
   auto issue = [&](int grp) {  // thread 0 only
     if (grp >= ngroups) return;
@@ -92,12 +94,8 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
     const int row = grp * G + g;
     double2 z[8];
     if constexpr (SWEEP) {
-      const int irow = (row + M) & (N - 1);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const int j = (2 * (t + r * TT) + M) & (N - 1);
-        z[r] = make_double2(sweep_pixel(jb.I, jb.sp, N, irow, j), sweep_pixel(jb.I, jb.sp, N, irow, j + 1));
-      }
+      sweep_row<double, M, 8>(z, jb.I, jb.sp, row, t, reinterpret_cast<double*>(B0 + g * RS),
+                              !EVEN || row <= M);
     } else {
       // a wait that gives up (never expected) is reported, and the block ends:
       // its one copy in flight is the one it has waited for
@@ -136,10 +134,11 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
     }
     // Bin by bin with the G rows of the group side by side, so that neighbouring
     // lanes fill the sectors of a column of F1 (column-major: bin k of row i at
-    // F1[k N + i]); row gg's buffer lies (gg - g) RS from ours.
+    // F1[k LD + i]); row gg's buffer lies (gg - g) RS from ours.
     const fx2* in0 = in - g * RS;
     for (int o = threadIdx.x; o < bd.Kc * G; o += G * TT) {
       const int k = o / G, gg = o - k * G;
+      if (EVEN && grp * G + gg > M) continue;
       const fx2* x = in0 + gg * RS;
       fx2 zk, zmk;
       if (pruned) {
@@ -150,7 +149,7 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
       }
       const fx2 X2 = fx_r2c_unpack2(zk, zmk, ldg_tw(tw + k));
       const int q = row_q[gg];
-      F1[(size_t)k * N + grp * G + gg] =
+      F1[(size_t)k * LD + grp * G + gg] =
           q == INT_MAX ? make_double2(fx_nan(), fx_nan()) : make_double2(fx_to(X2.x, q - 1), fx_to(X2.y, q - 1));
     }
     __syncthreads();  // every read of the work buffers and scales is done
@@ -200,7 +199,7 @@ col_fx_kernel(const __grid_constant__ Jobs<ColJob<double>, K> jobs, const double
     const bool act = c < ncol;
     double2 z[8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) z[r] = act ? F1[(size_t)c * N + t + r * TT] : make_double2(0.0, 0.0);
+    for (int r = 0; r < 8; ++r) z[r] = act ? F1[f1_index(jb.even, N, c, t + r * TT)] : make_double2(0.0, 0.0);
     fx2 v[8];
     const FxScale sc = fx_load<TT>(z, v, red_max, red_sum);
     FxHead<N, 0>::run(v, A, B, t, tab);
@@ -252,7 +251,8 @@ cudaError_t launch_row_fx(const Jobs<RowJob<double>, K>& jb, int n, int scale, b
   if (e) return e;
   if (per_sm < 1) per_sm = 1;
   int x = (per_sm * current_device_sms() * (scale < 1 ? 1 : scale) + n - 1) / n;
-  if (x > S::N / S::SH::G) x = S::N / S::SH::G;
+  constexpr int rows = even_rows<double, SWEEP, BEAM>(S::N) ? S::M + 1 : S::N;
+  if (x > (rows + S::G - 1) / S::G) x = (rows + S::G - 1) / S::G;
   if (x < 1) x = 1;
   if (dep) return launch_dependent(kern, dim3(x, n), dim3(S::SH::threads), smem, st, jb, tw, err);
   kern<<<dim3(x, n), S::SH::threads, smem, st>>>(jb, tw, err);

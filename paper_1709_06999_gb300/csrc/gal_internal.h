@@ -68,18 +68,22 @@ template <typename T> struct Launch {
                            cudaStream_t st);
   // err: bit 2 is set if a staged copy's wait timed out (never expected);
   // beam: primary-beam tables of beam_table (null: no beam); radix: values per
-  // thread of the compile-time FFT stages (0: the default, fft_radix_default)
+  // thread of the compile-time FFT stages (0: the default, fft_radix_default);
+  // kc_hint: window columns if the host knows them (0: unknown)
   static cudaError_t row_pass(const T* image, const T* I, const SweepParams& sp, int N,
                               const void* tw, void* F1, const double* rho2, double S, int* err,
-                              const T* beam, cudaStream_t st, int radix = 0);
+                              const T* beam, cudaStream_t st, int radix = 0, int kc_hint = 0);
   // primary-beam tables (2 N values) for a beam of FWHM fwhm > 0 on the
   // pointing centre, seen from a model moved by (dRA, dDec) at position angle PA
   static cudaError_t beam_table(T* tab, int N, double dxy, double fwhm, double dRA, double dDec,
                                 double PA, cudaStream_t st);
+  // whether row_pass keeps only rows 0 .. N/2 of a profile swept without a beam
+  static bool even_profile(int N);
   // kc_hint: window columns if the host knows them (0: unknown); full: the
-  // full-plane window of full_cols (lengths of the compile-time passes only)
+  // full-plane window of full_cols (lengths of the compile-time passes only);
+  // even: F1 comes from a row pass that kept half the rows (even_profile)
   static cudaError_t col_pass(const void* F1, void* Gw, int N, const void* tw,
-                              const double* rho2, double S, int kc_hint, bool full,
+                              const double* rho2, double S, int kc_hint, bool full, bool even,
                               cudaStream_t st, int radix = 0);
   // ms: multi-source offsets (null: the single offset of gp)
   static cudaError_t gather(const void* Gw, const GatherParams& gp, const double* rho2,
@@ -184,9 +188,9 @@ template <typename T> struct BatchLaunch {
 template <typename T>
 cudaError_t row_fft3(const T* image, const T* I, const SweepParams& sp, int N, const void* tw,
                      void* F1, const double* rho2, double S, int* err, const T* beam,
-                     cudaStream_t st, int radix);
+                     cudaStream_t st, int radix, int kc);
 template <typename T>
 cudaError_t col_fft3(const void* F1, void* Gw, int N, const void* tw, const double* rho2, double S,
-                     int kc_hint, bool full, cudaStream_t st, int radix);
+                     int kc_hint, bool full, bool even, cudaStream_t st, int radix);
 
 }  // namespace gal

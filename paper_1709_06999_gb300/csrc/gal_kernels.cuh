@@ -223,6 +223,37 @@ __global__ void sweep_kernel(const T* __restrict__ I, SweepT<T> p, int N, T* __r
   }
 }
 
+// Row `row` of the fftshifted sweep as the pixel pairs z_m = (x_{2m}, x_{2m+1})
+// of the real-to-complex row pass, thread t of TT holding pairs m = t + r TT.
+// The profile depends on |N/2 - j| only, so x_n = x_{N-n} bit for bit: pairs up
+// to the middle are evaluated, the others read back from `xs` (N/2 + 1 values of
+// scratch in shared memory; the caller's block synchronises here once).
+template <typename T, int M, int V>
+__device__ __forceinline__ void sweep_row(cplx_t<T> (&z)[V], const T* __restrict__ I,
+                                          const SweepT<T>& sp, int row, int t, T* xs, bool act) {
+  constexpr int N = 2 * M, TT = M / V;
+  const int irow = (row + M) & (N - 1);
+  if constexpr (V < 2) {
+    z[0] = mkc((T)0, (T)0);
+  } else {
+    if (act) {
+#pragma unroll
+      for (int r = 0; r < V / 2; ++r) {
+        const int m = t + r * TT;  // shifted columns 2 m < N/2: image columns 2 m + N/2
+        z[r] = mkc(sweep_pixel(I, sp, N, irow, 2 * m + M), sweep_pixel(I, sp, N, irow, 2 * m + 1 + M));
+        reinterpret_cast<cplx_t<T>*>(xs)[m] = z[r];
+      }
+      if (t == 0) xs[M] = sweep_pixel(I, sp, N, irow, 0);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = V / 2; r < V; ++r) {
+      const int m = t + r * TT;
+      z[r] = act ? mkc(xs[N - 2 * m], xs[N - 2 * m - 1]) : mkc((T)0, (T)0);
+    }
+  }
+}
+
 // Primary-beam tables (Sect. 2.1: A is the antenna pattern normalised at the
 // pointing centre, its central lobe a Gaussian of full width at half maximum
 // K lambda / D): A(s) = exp(-c |s|^2), c = 4 ln 2 / fwhm^2, fixed on the
@@ -385,6 +416,20 @@ template <typename C> __device__ __forceinline__ C r2c_unpack(C zk, C zmk, C w) 
   return cadd(e, cmul(cmul_mi(d), w));
 }
 
+// The passes keep rows 0 .. N/2 of a swept image (its row N - i is its row i)
+// where the compile-time column pass can mirror them, unless a beam breaks the
+// symmetry; kEvenRows: values kept to a column, whole 64-byte lines.
+template <typename T> constexpr int max_col_lg() { return sizeof(T) == 4 ? 13 : 12; }
+template <typename T, bool SWEEP, bool BEAM> constexpr bool even_rows(int N) {
+  return SWEEP && !BEAM && N / 2 >= FftV<T>::V && N <= (1 << max_col_lg<T>());
+}
+__host__ __device__ constexpr int kEvenRows(int N) { return N / 2 + 8; }
+
+// row i of column c of F1
+__device__ __forceinline__ size_t f1_index(int even, int N, int c, int i) {
+  return even ? (size_t)c * kEvenRows(N) + min(i, N - i) : (size_t)c * N + i;
+}
+
 // Launch shape of the length-L passes: G sequences per block (at least 128
 // threads), each with a shared-memory region of RS complex (padded, rounded
 // to 16 bytes so that bulk copies into it stay aligned).
@@ -445,6 +490,8 @@ row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>
   const double S = jb.S;
   const T* __restrict__ beam = BEAM ? jb.beam : nullptr;
   constexpr int M = 1 << LG, N = 2 * M;
+  constexpr bool EVEN = even_rows<T, SWEEP, BEAM>(N);
+  constexpr int LD = EVEN ? kEvenRows(N) : N;  // rows of F1 kept to a column
   using SH = Shape3<T, M, N, MINT, VR>;
   using P = typename SH::P;
   constexpr int V = SH::V, TT = P::T, G = SH::G, RS = SH::RS;
@@ -469,18 +516,19 @@ row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>
   auto transform = [&](C (&v)[V], C* A, C* B, int row) {
     Head3<M, V, 0>::run(v, A, B, t, tws, tw1, sync);
     C* in = last_input<M, V>(A, B);
-    C* out = F1 + row;  // column-major: bin j of this row at out[j N]
+    C* out = F1 + row;  // column-major: bin j of this row at out[j LD]
     if (pruned) {
+      if (EVEN && row > M) return;
       for (int j = t; j < bd.Kc; j += TT) {
         C zj, zmj;
         if (one_j) {
           pruned_pair3<M, V>(in, j, twp, zj, zmj);
-          out[(size_t)j * N] = r2c_unpack(zj, zmj, wj);
+          out[(size_t)j * LD] = r2c_unpack(zj, zmj, wj);
         } else {
           C tj[V];
           load_twp<M, V>(tj, j, tws);
           pruned_pair3<M, V>(in, j, tj, zj, zmj);
-          out[(size_t)j * N] = r2c_unpack(zj, zmj, __ldg(tw + j));
+          out[(size_t)j * LD] = r2c_unpack(zj, zmj, __ldg(tw + j));
         }
       }
     } else {
@@ -497,7 +545,8 @@ row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>
       for (int q = threadIdx.x; q < bd.Kc * G; q += G * TT) {
         const int k = q / G, gg = q - k * G;
         const C* og = o0 + (size_t)gg * RS;
-        out0[(size_t)k * N + gg] =
+        if (!EVEN || row - g + gg <= M)
+          out0[(size_t)k * LD + gg] =
             r2c_unpack(og[pad3<V>(k & (M - 1))], og[pad3<V>((M - k) & (M - 1))], __ldg(tw + k));
       }
     }
@@ -557,21 +606,27 @@ row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>
       if (threadIdx.x == 0) issue(it + NSLOT);
     }
   } else {
+    // a sweep without a beam is even in the rows too: row N - i is row i, so only
+    // rows 0 .. N/2 are transformed and kept (the column pass mirrors them)
     C* A = base + (size_t)g * RS;
     C* B = base + (size_t)(G + g) * RS;
     const int row = blockIdx.x * G + g;
-    const int irow = (row + M) & (N - 1);
+    const bool act = !EVEN || row <= M;
     if constexpr (BEAM) grid_dep_wait();  // the beam tables
     C v[V];
+    if constexpr (SWEEP) {
+      sweep_row<T, M, V>(v, I, sp, row, t, reinterpret_cast<T*>(B), act);
+    } else {
+      const int irow = (row + M) & (N - 1);
 #pragma unroll
-    for (int r = 0; r < V; ++r) {
-      const int n = t + r * TT;
-      const int j = (2 * n + M) & (N - 1);
-      if constexpr (SWEEP)
-        v[r] = mkc(sweep_pixel(I, sp, N, irow, j), sweep_pixel(I, sp, N, irow, j + 1));
-      else
+      for (int r = 0; r < V; ++r) {
+        const int j = (2 * (t + r * TT) + M) & (N - 1);
         v[r] = *reinterpret_cast<const C*>(image + (size_t)irow * N + j);
-      if constexpr (BEAM) v[r] = beam_pair(v[r], beam, N, row, n);
+      }
+    }
+    if constexpr (BEAM) {
+#pragma unroll
+      for (int r = 0; r < V; ++r) v[r] = beam_pair(v[r], beam, N, row, t + r * TT);
     }
     transform(v, A, B, row);
   }
@@ -803,7 +858,7 @@ col_fft3_kernel(const __grid_constant__ Jobs<ColJob<T>, K> jobs, const cplx_t<T>
     const bool act = c < ncol;
     C v[V];
 #pragma unroll
-    for (int r = 0; r < V; ++r) v[r] = act ? F1[(size_t)c * N + t + r * TT] : mkc((T)0, (T)0);
+    for (int r = 0; r < V; ++r) v[r] = act ? F1[f1_index(jb.even, N, c, t + r * TT)] : mkc((T)0, (T)0);
     Head3<N, V, 0>::run(v, A, B, t, tws, tw1, sync);
     C* in = last_input<N, V>(A, B);
     if (pruned) {
@@ -934,7 +989,9 @@ template <typename T> struct ColJob {
   const double* rho2;
   double S;
   int full;             // 1: the full-plane window (full_cols(bd, N).W columns)
+  int even;             // 1: F1 holds rows 0 .. N/2 only, row N - i being row i
 };
+
 
 template <> struct GatherT<double> {
   double A, B, phx, phy;  // A = cos(PA) N dxy, B = sin(PA) N dxy, as for float
@@ -1977,12 +2034,12 @@ cudaError_t Launch<T>::sweep(const T* I, const SweepParams& sp, int N, T* img, i
 template <typename T>
 cudaError_t Launch<T>::row_pass(const T* image, const T* I, const SweepParams& sp, int N,
                                 const void* tw, void* F1, const double* rho2, double S, int* err,
-                                const T* beam, cudaStream_t st, int radix) {
+                                const T* beam, cudaStream_t st, int radix, int kc_hint) {
   using C = cplx_t<T>;
   const int M = N / 2;
   const bool al16 = I || (reinterpret_cast<uintptr_t>(image) & 15u) == 0;
   if (M >= FftV<T>::V && al16) {
-    const cudaError_t e = row_fft3<T>(image, I, sp, N, tw, F1, rho2, S, err, beam, st, radix);
+    const cudaError_t e = row_fft3<T>(image, I, sp, N, tw, F1, rho2, S, err, beam, st, radix, kc_hint);
     if (e != cudaErrorNotSupported) return e;
   }
   const C* twc = static_cast<const C*>(tw);
@@ -2014,15 +2071,20 @@ cudaError_t Launch<T>::beam_table(T* tab, int N, double dxy, double fwhm, double
 }
 
 template <typename T>
+bool Launch<T>::even_profile(int N) {
+  return even_rows<T, true, false>(N);
+}
+
+template <typename T>
 cudaError_t Launch<T>::col_pass(const void* F1, void* Gw, int N, const void* tw,
-                                const double* rho2, double S, int kc_hint, bool full,
+                                const double* rho2, double S, int kc_hint, bool full, bool even,
                                 cudaStream_t st, int radix) {
   using C = cplx_t<T>;
   if (N >= FftV<T>::V) {
-    const cudaError_t e = col_fft3<T>(F1, Gw, N, tw, rho2, S, kc_hint, full, st, radix);
+    const cudaError_t e = col_fft3<T>(F1, Gw, N, tw, rho2, S, kc_hint, full, even, st, radix);
     if (e != cudaErrorNotSupported) return e;
   }
-  if (full) return cudaErrorNotSupported;  // the generic pass keeps the half plane only
+  if (full || even) return cudaErrorNotSupported;  // the generic pass keeps the half plane, whole
   const int P = N / 2 + 1;
   const int tg = col_threads_per_col(N);
   int cpb = 256 / tg;

@@ -126,7 +126,7 @@ extern "C" int gal_chi2_image_noalloc_f32(const float* image, int nxy, double dx
   if (gal::Launch<float>::row_pass(image, nullptr, none, nxy, tw, F1, rho2, S, err, nullptr, cs,
                                    rv) != cudaSuccess)
     return GAL_E_CUDA;
-  if (gal::Launch<float>::col_pass(F1, Gw, nxy, tw, rho2, S, 0, false, cs, cv) != cudaSuccess)
+  if (gal::Launch<float>::col_pass(F1, Gw, nxy, tw, rho2, S, 0, false, false, cs, cv) != cudaSuccess)
     return GAL_E_CUDA;
   gal::GatherParams gp;
   gp.cpa = std::cos(PA);
