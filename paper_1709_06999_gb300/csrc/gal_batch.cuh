@@ -151,7 +151,8 @@ cudaError_t gather(const BatchItem* it, const int* idx, int n, int grid, int fol
   }
   if (!SMEM) smem = 0;
   constexpr auto kern = gather_kernel<T, true, SMEM, EDGE, kBatchJobs, false, FULL>;
-  const cudaError_t e = ensure_smem_attr<kern>(smem);
+  const cudaError_t e =
+      SMEM ? ensure_smem_attr<kern>(smem) : ensure_l1_carveout<T, kern>();
   if (e) return e;
   const int threads = gather_threads<T, SMEM, FULL>();
   if (fold_max < 1) fold_max = 1;

@@ -1895,6 +1895,29 @@ template <auto Kern> cudaError_t ensure_smem_attr(size_t smem) {
   return e;
 }
 
+// Ask for the split of an SM's memory that leaves float gather `kern` the most
+// L1 (a hint, per device; set once).  A gather that reads its window through L1
+// starts, as a programmatic dependent, on SMs that the row and column passes have
+// set to their large shared memory, and without the hint it keeps that split for
+// its whole run: four copies of a 2048 / 2e6 model 65 -> 40 us, an 8192 image with
+// 5e6 points and a beam 388 -> 289 us, 2e6 samples of a 1024 image 72 -> 57 us, all
+// for the whole call (launched as an ordinary successor instead: 44, 291 and 60 us,
+// and 4 us more where a call is small).  The double gather has its table in shared
+// memory and gained nothing (84.2 against 84.5 us, 99.0 against 99.4), so it is
+// left to the default.
+template <typename T, auto Kern> cudaError_t ensure_l1_carveout() {
+  if (sizeof(T) == 8) return cudaSuccess;
+  constexpr int kDev = 64, kPercent = 4;  // of 228 KB: the blocks' reduction scratch
+  static std::atomic<bool> done[kDev] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e) return e;
+  if (dev < 0 || dev >= kDev || done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+  e = cudaFuncSetAttribute(Kern, cudaFuncAttributePreferredSharedMemoryCarveout, kPercent);
+  if (e == cudaSuccess) done[dev].store(true, std::memory_order_relaxed);
+  return e;
+}
+
 // Launch `kern` as a programmatic dependent of the preceding kernel in `st`:
 // it may be scheduled while that kernel finishes, and waits for it in
 // grid_dep_wait() before reading what it wrote.
@@ -2130,14 +2153,14 @@ cudaError_t Launch<T>::gather(const void* Gw, const GatherParams& gp, const doub
     const size_t smem = SM ? window_smem : 0;
     if (ms && ms->K > 0) {
       constexpr auto kern = gather_kernel<T, CH, SM, ED, 1, true>;
-      le = ensure_smem_attr<kern>(smem);
+      le = SM ? ensure_smem_attr<kern>(smem) : ensure_l1_carveout<T, kern>();
       MultiArg<T, true> ma;
       ma.m = MultiPhase<T>::make(ms->K, ms->dRA, ms->dDec, ms->amp);
       if (le == cudaSuccess)
         le = launch_dependent(kern, dim3(grid), dim3(threads), smem, st, jb, nodes, ma);
     } else {
       constexpr auto kern = gather_kernel<T, CH, SM, ED, 1, false>;
-      le = ensure_smem_attr<kern>(smem);
+      le = SM ? ensure_smem_attr<kern>(smem) : ensure_l1_carveout<T, kern>();
       if (le == cudaSuccess)
         le = launch_dependent(kern, dim3(grid), dim3(threads), smem, st, jb, nodes,
                               MultiArg<T, false>{});

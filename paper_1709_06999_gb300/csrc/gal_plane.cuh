@@ -355,7 +355,7 @@ cudaError_t Plane<T>::gather(const void* Gw, const GatherParams& gp, const doubl
                    ED = decltype(edge_c)::value;
     constexpr auto kern = gather_kernel<T, CH, SM, ED, 1, false, true>;
     const size_t smem = SM ? window_smem : 0;
-    le = ensure_smem_attr<kern>(smem);
+    le = SM ? ensure_smem_attr<kern>(smem) : ensure_l1_carveout<T, kern>();
     if (le == cudaSuccess)
       le = launch_dependent(kern, dim3(grid), dim3(threads), smem, st, jb, nodes,
                             MultiArg<T, false>{});
