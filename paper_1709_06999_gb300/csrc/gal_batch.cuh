@@ -126,8 +126,9 @@ cudaError_t cols(const BatchItem* it, const int* idx, int n, const void* tw, cud
   }
 }
 
-// Each request keeps the block partition of its single call (`grid` virtual
-// blocks, one partial sum each); a launch of n requests runs min(n, fold) of
+// Each request keeps the block partition of its single call (gather_vblocks of
+// `grid` virtual blocks, one partial sum each; a launch holds requests of any
+// number of points); a launch of n requests runs min(n, fold) of
 // them per block in turn (fold from the launch shape, kGatherFold by
 // default), so a request's window is copied by that many times fewer blocks
 // while the launch still fills the GPU (a launch of one request runs its
@@ -139,6 +140,8 @@ cudaError_t gather(const BatchItem* it, const int* idx, int n, int grid, int fol
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   Jobs<GatherJob<T>, kBatchJobs> jb{};
   size_t smem = 0;
+  const int threads = gather_threads<T, SMEM, FULL>();
+  int vmax = 1;
   for (int k = 0; k < n; ++k) {
     const BatchItem& b = it[idx[k]];
     const int vec = al16(b.u) && al16(b.v) && al16(b.re) && al16(b.im) && al16(b.w);
@@ -146,7 +149,8 @@ cudaError_t gather(const BatchItem* it, const int* idx, int n, int grid, int fol
                            static_cast<const T*>(b.u), static_cast<const T*>(b.v),
                            static_cast<const T*>(b.re), static_cast<const T*>(b.im),
                            static_cast<const T*>(b.w), b.M, vec, nullptr, b.partials,
-                           b.counter, b.chi2_out, grid};
+                           b.counter, b.chi2_out, gather_vblocks<T>(grid, b.M, vec, threads)};
+    vmax = jb.j[k].vblocks > vmax ? jb.j[k].vblocks : vmax;
     smem = b.wbytes > smem ? b.wbytes : smem;
   }
   if (!SMEM) smem = 0;
@@ -154,11 +158,10 @@ cudaError_t gather(const BatchItem* it, const int* idx, int n, int grid, int fol
   const cudaError_t e =
       SMEM ? ensure_smem_attr<kern>(smem) : ensure_l1_carveout<T, kern>();
   if (e) return e;
-  const int threads = gather_threads<T, SMEM, FULL>();
   if (fold_max < 1) fold_max = 1;
   if (fold_max > kMaxGatherFold) fold_max = kMaxGatherFold;
   const int fold = n < fold_max ? n : fold_max;
-  const int blocks = (grid + fold - 1) / fold;
+  const int blocks = (vmax + fold - 1) / fold;
   kern<<<dim3(blocks, n), threads, smem, st>>>(jb, (int)(smem / sizeof(C)), MultiArg<T, false>{});
   return cudaGetLastError();
 }

@@ -340,12 +340,7 @@ cudaError_t Plane<T>::gather(const void* Gw, const GatherParams& gp, const doubl
   if (chi2) vec = vec && al16(re) && al16(im) && al16(w);
   const int nodes = (int)(window_smem / sizeof(C));
   const int threads = window_smem ? gather_threads<T, true, true>() : gather_threads<T, false, true>();
-  int grid = blocks;
-  if (!chi2) {
-    int64_t need = (M + threads - 1) / threads;
-    if (need < 1) need = 1;
-    if (need < grid) grid = (int)need;
-  }
+  const int grid = gather_vblocks<T>(blocks, M, chi2 ? vec : 0, threads);
   Jobs<GatherJob<T>, 1> jb;
   jb.j[0] = GatherJob<T>{static_cast<const C*>(Gw), GatherT<T>::make(gp), rho2, u, v, re, im, w, M,
                          vec, static_cast<C*>(vis), partials, counter, chi2};
