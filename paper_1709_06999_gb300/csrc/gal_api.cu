@@ -312,11 +312,8 @@ template <typename T> int reserve_call(gal_ctx* ctx, int nxy, const CallOpts& o)
 // which one runs.  There is one plan per device, side and precision for the
 // whole process, so single calls, batches, served requests and the
 // allocation-free entry point compute a request with the same arithmetic
-// (bitwise equal results).  A side's plan is fixed at its first use on a
-// context: timed on that context's workspace and stream when its tuning is on
-// and the stream is not being captured (each radix, each pass, best of three,
-// the smaller radix kept only when at least 5 % faster), otherwise the
-// default; gal_set_fft_radix overrides it.
+// (bitwise equal results): that of fft_radix_default, the same in every
+// process, unless gal_set_fft_radix overrides it.
 // ---------------------------------------------------------------------------
 namespace plans {
 constexpr int kDevices = 64;
@@ -328,9 +325,9 @@ template <typename T> bool plan_tunable(int nxy) {
   return sizeof(T) == 4 && nxy >= 32 && nxy <= gal::kAltRadixMaxSide;
 }
 
-// the plan of side nxy on `device` if chosen (returns false and the defaults otherwise)
+// the plan of side nxy on `device` if set or used (returns false and the defaults otherwise)
 template <typename T> bool plan_lookup(int device, int nxy, int* rv, int* cv) {
-  *rv = *cv = gal::fft_radix_default<T>();
+  gal::fft_radix_default<T>(nxy, rv, cv);
   if (device < 0 || device >= plans::kDevices || !plan_tunable<T>(nxy)) return true;
   std::lock_guard<std::mutex> lk(plans::mu);
   const int* e = plans::table[device][prec_index<T>()][log2i(nxy)];
@@ -349,61 +346,10 @@ template <typename T> void plan_store(int device, int nxy, int rv, int cv, bool 
   e[1] = cv;
 }
 
-// Time both radices of the row and column passes of side nxy on the
-// context's own workspace (its contents serve as input: only the time
-// matters) with the uv extent of the whole half spectrum.
-template <typename T> int tune_fft(gal_ctx* ctx, int nxy, cudaStream_t st, int* rv, int* cv) {
-  GAL_TRY(ensure<T>(ctx, nxy));
-  const void* tw = ctx->tw[prec_index<T>()][log2i(nxy)];
-  const double big = 1e300;  // beyond any grid: nothing is pruned
-  GAL_CUDA(ctx, cudaMemcpyAsync(ctx->rho2, &big, sizeof(double), cudaMemcpyHostToDevice, st));
-  const T* img = static_cast<const T*>(ctx->Gw);
-  const double S = 1.0;
-  cudaEvent_t a = pool_event(ctx), b = pool_event(ctx);
-  auto best_of = [&](auto&& launch, float* ms) -> int {
-    *ms = 1e30f;
-    for (int rep = 0; rep < 3; ++rep) {
-      GAL_CUDA(ctx, cudaEventRecord(a, st));
-      GAL_CUDA(ctx, launch());
-      ctx->launches++;
-      GAL_CUDA(ctx, cudaEventRecord(b, st));
-      GAL_CUDA(ctx, cudaEventSynchronize(b));
-      float t = 0.f;
-      GAL_CUDA(ctx, cudaEventElapsedTime(&t, a, b));
-      if (rep > 0 && t < *ms) *ms = t;  // the first run warms up
-    }
-    return GAL_OK;
-  };
-  const int r0 = gal::fft_radix_default<T>(), r1 = gal::kAltRadix;
-  float row[2], col[2];
-  for (int k = 0; k < 2; ++k) {
-    const int r = k ? r1 : r0;
-    GAL_TRY(best_of([&] {
-      return gal::Launch<T>::row_pass(img, nullptr, gal::SweepParams{}, nxy, tw, ctx->F1, ctx->rho2,
-                                      S, ctx->err, nullptr, st, r);
-    }, &row[k]));
-    GAL_TRY(best_of([&] {
-      return gal::Launch<T>::col_pass(ctx->F1, ctx->Gw, nxy, tw, ctx->rho2, S, 0, false, false, st, r);
-    }, &col[k]));
-  }
-  ctx->event_pool.push_back(a);
-  ctx->event_pool.push_back(b);
-  *rv = row[1] < 0.95f * row[0] ? r1 : r0;
-  *cv = col[1] < 0.95f * col[0] ? r1 : r0;
-  return GAL_OK;
-}
-
-// Fix (or look up) the plan of side nxy before a call enqueues anything.
-template <typename T> int fft_plan(gal_ctx* ctx, int nxy, cudaStream_t st) {
+// Fix the plan of side nxy at its first use.
+template <typename T> void fft_plan(gal_ctx* ctx, int nxy) {
   int rv, cv;
-  if (plan_lookup<T>(ctx->device, nxy, &rv, &cv)) return GAL_OK;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  GAL_CUDA(ctx, cudaStreamIsCapturing(st, &cap));
-  rv = cv = gal::fft_radix_default<T>();
-  if (ctx->batch_tuning && cap == cudaStreamCaptureStatusNone)
-    GAL_TRY(tune_fft<T>(ctx, nxy, st, &rv, &cv));
-  plan_store<T>(ctx->device, nxy, rv, cv, false);
-  return GAL_OK;
+  if (!plan_lookup<T>(ctx->device, nxy, &rv, &cv)) plan_store<T>(ctx->device, nxy, rv, cv, false);
 }
 
 // FFT of the image (or of the swept profile) into the pruned window ctx->Gw;
@@ -443,7 +389,7 @@ int sample_impl(gal_ctx* ctx, const T* image, const T* I, const gal::SweepParams
   if (!aligned(u, sizeof(T)) || !aligned(v, sizeof(T)) || !aligned(vis, 2 * sizeof(T)))
     return GAL_E_INVAL;
   GAL_TRY(reserve_call<T>(ctx, nxy, o));
-  GAL_TRY(fft_plan<T>(ctx, nxy, st));
+  fft_plan<T>(ctx, nxy);
   GAL_TRY(stage(ctx, 0, st, [&] {
     return gal::Launch<T>::extent(u, v, M, ctx->rho2, ctx->aux_blocks, st);
   }));
@@ -504,7 +450,7 @@ int chi2_impl(gal_ctx* ctx, const T* image, const T* I, const gal::SweepParams& 
   }
   using C = gal::cplx_t<T>;
   GAL_TRY(reserve_call<T>(ctx, nxy, o));
-  GAL_TRY(fft_plan<T>(ctx, nxy, st));
+  fft_plan<T>(ctx, nxy);
   const gal::Bounds bd = gal::make_bounds(d->rho2_host, (double)nxy * dxy, nxy);
   const T* beam;
   GAL_TRY(beam_tables<T>(ctx, o, nxy, dxy, dRA, dDec, PA, st, &beam));
@@ -1161,7 +1107,7 @@ int run_batch(gal_ctx* ctx, const gal_request* reqs, int n, double* chi2_out, cu
   if (allow_setup) {
     for (const auto& b : pl.items[0]) GAL_TRY(ensure_tables<float>(ctx, b.N));
     for (const auto& b : pl.items[1]) GAL_TRY(ensure_tables<double>(ctx, b.N));
-    for (const auto& b : pl.items[0]) GAL_TRY(fft_plan<float>(ctx, b.N, st));
+    for (const auto& b : pl.items[0]) fft_plan<float>(ctx, b.N);
   }
   // every request runs with the FFT plan of its side (the same as a single call's)
   for (auto& b : pl.items[0]) plan_lookup<float>(ctx->device, b.N, &b.radix_row, &b.radix_col);

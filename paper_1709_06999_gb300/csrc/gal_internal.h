@@ -68,7 +68,7 @@ template <typename T> struct Launch {
                            cudaStream_t st);
   // err: bit 2 is set if a staged copy's wait timed out (never expected);
   // beam: primary-beam tables of beam_table (null: no beam); radix: values per
-  // thread of the compile-time FFT stages (0: the default, fft_radix_default);
+  // thread of the compile-time FFT stages (kAltRadix, or any other value for FftV);
   // kc_hint: window columns if the host knows them (0: unknown)
   static cudaError_t row_pass(const T* image, const T* I, const SweepParams& sp, int N,
                               const void* tw, void* F1, const double* rho2, double S, int* err,
@@ -116,14 +116,26 @@ template <typename T> struct Plane {
 constexpr int kBatchJobs = 32;
 
 // FFT radix (values per thread of every stage but the last) of the
-// compile-time row and column passes.  Float transforms run at radix 16; for
-// image sides up to kAltRadixMaxSide the radix-8 passes exist too, and the
-// FFT plan (a per-device choice per side, see gal_set_fft_radix) says which
-// of the two a call uses.  Double transforms always run at radix 8.
-template <typename T> constexpr int fft_radix_default() { return sizeof(T) == 4 ? 16 : 8; }
+// compile-time row and column passes.  Double transforms run at radix 8, float
+// ones at radix 16; for float image sides 32 .. kAltRadixMaxSide the radix-8
+// passes exist too, and the plan of the side (gal_set_fft_radix) says which a
+// call uses.
 constexpr int kAltRadix = 8;
 constexpr int kAltRadixMaxSide = 512;
-// the FFT plan of a float32 side on `device` if one is fixed, the defaults
+// Default plan.  Short float columns run at radix 8: twice the threads to a
+// column (side 512: 27 against 33 us for 32 unpruned images in a batch, 7.8
+// against 10.9 for one; level or better down to 32 but for batches of side 256,
+// 12.9 against 10.9).  Rows run at radix 8 where it takes no more stages than
+// radix 16, i.e. for 32 and 64 complex points, sides 64 and 128 (12.0 against
+// 14.2 and 11.8 against 14.1 us for 32 images), and at 16 elsewhere (side 512:
+// 23 against 28 us).  A rule, not a timing in each process, because the two
+// round differently: results are the same in every process.
+template <typename T> inline void fft_radix_default(int nxy, int* row, int* col) {
+  const bool alt = sizeof(T) == 4 && nxy >= 32 && nxy <= kAltRadixMaxSide;
+  *col = sizeof(T) == 8 || alt ? 8 : 16;
+  *row = sizeof(T) == 8 || (alt && (nxy == 64 || nxy == 128)) ? 8 : 16;
+}
+// the FFT plan of a float32 side on `device` if one is set, the default
 // otherwise (fixes nothing; for callers without a context)
 void fft_plan_lookup_f32(int device, int nxy, int* rv, int* cv);
 
