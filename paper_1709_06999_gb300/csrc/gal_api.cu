@@ -48,6 +48,8 @@ struct gal_ctx {
   int partials_len = 0;
   unsigned* counter = nullptr;  // last-block-done counter (self-resetting)
   double* rho2 = nullptr;       // uv extent scratch for raw-pointer calls
+  void* ext_state = nullptr;    // Launch::extent's: of those calls, and of registrations
+  double* reg_rho2 = nullptr;   // extent of the observation being registered (mapped host memory)
   double* uvrange = nullptr;    // min / max of u^2 + v^2 (image sizing)
   int* err = nullptr;           // index-check flag
   double* chi2_dev = nullptr;   // result slot for the host-buffer entry points
@@ -92,8 +94,7 @@ struct gal_data {
   int real_bytes = 0;
   int64_t M = 0;
   const void *u = nullptr, *v = nullptr, *re = nullptr, *im = nullptr, *w = nullptr;
-  double* rho2 = nullptr;  // device scalar: max(u^2 + v^2)
-  double rho2_host = 0.0;  // the same value, read back once at registration
+  double rho2_host = 0.0;  // max(u^2 + v^2), read back once at registration
   void* uv_own = nullptr;  // arrays the handle owns: u, v in wavelengths when registered
                            // from metres, or all five when registered in Z-order
 };
@@ -356,7 +357,7 @@ template <typename T> void fft_plan(gal_ctx* ctx, int nxy) {
 // `beam` multiplies the pixels (null: none), `full` keeps both signs of u.
 template <typename T>
 int spectrum(gal_ctx* ctx, const T* image, const T* I, const gal::SweepParams& sp, int nxy,
-             double dxy, const double* rho2, int kc_hint, cudaStream_t st,
+             double dxy, const gal::UvExtent& rho2, int kc_hint, cudaStream_t st,
              const T* beam = nullptr, bool full = false) {
   GAL_TRY(ensure<T>(ctx, nxy, full));
   const void* tw = ctx->tw[prec_index<T>()][log2i(nxy)];
@@ -391,22 +392,23 @@ int sample_impl(gal_ctx* ctx, const T* image, const T* I, const gal::SweepParams
   GAL_TRY(reserve_call<T>(ctx, nxy, o));
   fft_plan<T>(ctx, nxy);
   GAL_TRY(stage(ctx, 0, st, [&] {
-    return gal::Launch<T>::extent(u, v, M, ctx->rho2, ctx->aux_blocks, st);
+    return gal::Launch<T>::extent(u, v, M, ctx->rho2, ctx->ext_state, ctx->num_sms, st);
   }));
+  const gal::UvExtent ext{ctx->rho2, gal::Bounds{}};
   const T* beam;
   GAL_TRY(beam_tables<T>(ctx, o, nxy, dxy, dRA, dDec, PA, st, &beam));
-  GAL_TRY(spectrum<T>(ctx, image, I, sp, nxy, dxy, ctx->rho2, 0, st, beam, o.full));
+  GAL_TRY(spectrum<T>(ctx, image, I, sp, nxy, dxy, ext, 0, st, beam, o.full));
   const gal::GatherParams gp = gather_params(ctx, nxy, dxy, dRA, dDec, PA);
   if (o.full) {
     const int blocks = ctx->num_sms * gal::Plane<T>::gather_blocks_per_sm(false, 0);
     return stage(ctx, 3, st, [&] {
-      return gal::Plane<T>::gather(ctx->Gw, gp, ctx->rho2, u, v, nullptr, nullptr, nullptr, M,
+      return gal::Plane<T>::gather(ctx->Gw, gp, ext, u, v, nullptr, nullptr, nullptr, M,
                                    vis, nullptr, nullptr, nullptr, 0, true, blocks, st);
     });
   }
   const int blocks = ctx->gather_blocks[prec_index<T>()][0];
   return stage(ctx, 3, st, [&] {
-    return gal::Launch<T>::gather(ctx->Gw, gp, ctx->rho2, u, v, nullptr, nullptr, nullptr, M,
+    return gal::Launch<T>::gather(ctx->Gw, gp, ext, u, v, nullptr, nullptr, nullptr, M,
                                   vis, nullptr, nullptr, nullptr, 0, true, blocks, ms, st);
   });
 }
@@ -452,29 +454,30 @@ int chi2_impl(gal_ctx* ctx, const T* image, const T* I, const gal::SweepParams& 
   GAL_TRY(reserve_call<T>(ctx, nxy, o));
   fft_plan<T>(ctx, nxy);
   const gal::Bounds bd = gal::make_bounds(d->rho2_host, (double)nxy * dxy, nxy);
+  const gal::UvExtent ext{nullptr, bd};
   const T* beam;
   GAL_TRY(beam_tables<T>(ctx, o, nxy, dxy, dRA, dDec, PA, st, &beam));
   const gal::GatherParams gp = gather_params(ctx, nxy, dxy, dRA, dDec, PA);
   if (o.full) {
     const int W = gal::full_cols(bd, nxy).W;
-    GAL_TRY(spectrum<T>(ctx, image, I, sp, nxy, dxy, d->rho2, W, st, beam, true));
+    GAL_TRY(spectrum<T>(ctx, image, I, sp, nxy, dxy, ext, W, st, beam, true));
     size_t wbytes = ((size_t)bd.nrw * W * sizeof(C) + 15) & ~size_t(15);  // bulk-copy size
     if (wbytes > kWindowSmem) wbytes = 0;
     int blocks = ctx->num_sms * gal::Plane<T>::gather_blocks_per_sm(true, wbytes);
     if (blocks > ctx->partials_len) blocks = ctx->partials_len;
     return stage(ctx, 3, st, [&] {
-      return gal::Plane<T>::gather(ctx->Gw, gp, d->rho2, static_cast<const T*>(d->u),
+      return gal::Plane<T>::gather(ctx->Gw, gp, ext, static_cast<const T*>(d->u),
                                    static_cast<const T*>(d->v), static_cast<const T*>(d->re),
                                    static_cast<const T*>(d->im), static_cast<const T*>(d->w),
                                    d->M, nullptr, ctx->partials, ctx->counter, chi2, wbytes,
                                    /*edge=*/bd.r0 == 0, blocks, st);
     });
   }
-  GAL_TRY(spectrum<T>(ctx, image, I, sp, nxy, dxy, d->rho2, bd.Kc, st, beam));
+  GAL_TRY(spectrum<T>(ctx, image, I, sp, nxy, dxy, ext, bd.Kc, st, beam));
   size_t wbytes;
   const int blocks = chi2_gather_shape<T>(ctx, bd, &wbytes);
   return stage(ctx, 3, st, [&] {
-    return gal::Launch<T>::gather(ctx->Gw, gp, d->rho2, static_cast<const T*>(d->u),
+    return gal::Launch<T>::gather(ctx->Gw, gp, ext, static_cast<const T*>(d->u),
                                   static_cast<const T*>(d->v), static_cast<const T*>(d->re),
                                   static_cast<const T*>(d->im), static_cast<const T*>(d->w), d->M,
                                   nullptr, ctx->partials, ctx->counter, chi2, wbytes,
@@ -596,27 +599,24 @@ int data_create_t(gal_ctx* ctx, const T* u, const T* v, const T* re, const T* im
   d->re = re;
   d->im = im;
   d->w = w;
-  cudaError_t e = cudaMalloc(&d->rho2, sizeof(double));
-  if (e != cudaSuccess) {
-    delete d;
-    return cuda_fail(ctx, e);
-  }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int s = stage(ctx, 0, st, [&] {
-    return gal::Launch<T>::extent(u, v, M, d->rho2, ctx->aux_blocks, st);
-  });
-  if (s == GAL_OK) {
-    // one read-back at registration: the host sizes the gather's shared
-    // window from it (the kernels read the device copy)
-    cudaError_t e2 = cudaMemcpyAsync(&d->rho2_host, d->rho2, sizeof(double),
-                                     cudaMemcpyDeviceToHost, st);
-    if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(st);
-    if (e2 != cudaSuccess) s = cuda_fail(ctx, e2);
-  }
-  if (s != GAL_OK) {
-    cudaFree(d->rho2);
-    delete d;
-    return s;
+  if (M > 0) {
+    // the extent comes back once, into mapped host memory: every call sizes its
+    // window from it on the host and passes the kernels the result
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    int s = stage(ctx, 0, st, [&] {
+      return gal::Launch<T>::extent(u, v, M, ctx->reg_rho2,
+                                    static_cast<char*>(ctx->ext_state) + gal::kExtentState,
+                                    ctx->num_sms, st);
+    });
+    if (s == GAL_OK) {
+      const cudaError_t e = cudaStreamSynchronize(st);
+      if (e != cudaSuccess) s = cuda_fail(ctx, e);
+    }
+    if (s != GAL_OK) {
+      delete d;
+      return s;
+    }
+    d->rho2_host = *static_cast<volatile double*>(ctx->reg_rho2);
   }
   *out = d;
   return GAL_OK;
@@ -904,8 +904,8 @@ int plan_batch(gal_ctx* ctx, const gal_request* reqs, int n, double* chi2_out, B
     b.sp = gal::SweepParams{r.Rmin, r.dR, r.dxy, r.inc, r.nr};
     b.N = r.nxy;
     b.S = (double)r.nxy * r.dxy;
-    b.rho2 = d->rho2;
     const gal::Bounds bd = gal::make_bounds(d->rho2_host, b.S, r.nxy);
+    b.rho2 = gal::UvExtent{nullptr, bd};
     b.Kc = bd.Kc;
     b.nrw = bd.nrw;
     if (p) GAL_TRY(ensure_twiddles<double>(ctx, kSinCosLen));
@@ -1241,6 +1241,9 @@ int gal_create(gal_ctx** out, int device) {
   if (!e) e = cudaMalloc(&ctx->partials, sizeof(double) * (size_t)maxb);
   if (!e) e = cudaMalloc(&ctx->counter, sizeof(unsigned));
   if (!e) e = cudaMalloc(&ctx->rho2, sizeof(double));
+  if (!e) e = cudaMalloc(&ctx->ext_state, 2 * gal::kExtentState);
+  if (!e) e = cudaMemset(ctx->ext_state, 0, 2 * gal::kExtentState);
+  if (!e) e = cudaHostAlloc((void**)&ctx->reg_rho2, sizeof(double), cudaHostAllocMapped);
   if (!e) e = cudaMalloc(&ctx->uvrange, 2 * sizeof(double));
   if (!e) e = cudaMalloc(&ctx->err, sizeof(int));
   if (!e) e = cudaMalloc(&ctx->chi2_dev, sizeof(double));
@@ -1261,10 +1264,11 @@ void gal_destroy(gal_ctx* ctx) {
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
   for (void* p : {ctx->F1, ctx->Gw, (void*)ctx->partials, (void*)ctx->counter, (void*)ctx->rho2,
-                  (void*)ctx->uvrange, ctx->batch_ws, (void*)ctx->batch_ctr,
+                  (void*)ctx->uvrange, ctx->ext_state, ctx->batch_ws, (void*)ctx->batch_ctr,
                   (void*)ctx->err, (void*)ctx->chi2_dev, ctx->stage_img, ctx->beam,
                   ctx->pipe_img[0], ctx->pipe_img[1], (void*)ctx->pipe_chi2})
     if (p) cudaFree(p);
+  if (ctx->reg_rho2) cudaFreeHost(ctx->reg_rho2);
   for (cudaEvent_t e : {ctx->pipe_copied[0], ctx->pipe_copied[1], ctx->pipe_done[0],
                         ctx->pipe_done[1]})
     if (e) cudaEventDestroy(e);
@@ -1570,7 +1574,6 @@ int gal_data_info(const gal_data* d, int64_t* M_out, int* real_bytes_out) {
 void gal_data_destroy(gal_data* d) {
   if (!d) return;
   cudaDeviceSynchronize();
-  if (d->rho2) cudaFree(d->rho2);
   if (d->uv_own) cudaFree(d->uv_own);
   delete d;
 }

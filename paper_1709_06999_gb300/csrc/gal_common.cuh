@@ -150,12 +150,30 @@ __host__ __device__ __forceinline__ FullCols full_cols(const Bounds& b, int N) {
   return f;
 }
 
-// Bounds for the whole block: one thread evaluates them (FP64: GB300's FP64
-// pipe is narrow, so no per-thread FP64 work) and shares them.  Every thread
-// of the block must call it.
-__device__ __forceinline__ Bounds block_bounds(const double* rho2, double S, int N) {
+// The window of a call: known to the host (a registered observation, whose
+// extent was read back once), or from max(u^2 + v^2) that an extent pass earlier
+// in the stream leaves at `rho2`.
+struct UvExtent {
+  const double* rho2;  // device; null: bd holds
+  Bounds bd;
+};
+
+// Wait for the kernels this grid is a programmatic dependent of (a no-op
+// otherwise); every read of what they wrote comes after it.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Bounds for the whole block; every thread of the block must call it, and it
+// synchronises.  With a device extent it waits for the kernels this grid depends
+// on, and one thread evaluates the bounds (FP64: GB300's FP64 pipe is narrow, so
+// no per-thread FP64 work).
+__device__ __forceinline__ Bounds block_bounds(const UvExtent& e, double S, int N) {
+  if (!e.rho2) {
+    __syncthreads();
+    return e.bd;
+  }
   __shared__ Bounds sb;
-  if (threadIdx.x == 0) sb = make_bounds(*rho2, S, N);
+  grid_dep_wait();
+  if (threadIdx.x == 0) sb = make_bounds(*e.rho2, S, N);
   __syncthreads();
   return sb;
 }

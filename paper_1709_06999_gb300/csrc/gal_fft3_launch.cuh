@@ -39,22 +39,24 @@ template <typename T, int LG, bool SWEEP> constexpr bool row_pairs_exist() {
 }
 constexpr int kRowPairsKc = 256;  // spans of the pruned last stage of 4096 points
 
-// A row pass with a beam follows beam_table_kernel in the stream and is
-// launched as its programmatic dependent (BEAM kernels wait for the tables).
+// A row pass that follows beam_table_kernel in the stream, or the extent pass
+// whose result it reads, is launched as its programmatic dependent (the kernels
+// wait for the tables, and block_bounds for the extent).
 template <typename T, int LG, bool SWEEP, bool BEAM, int V = FftV<T>::V, bool PAIRS = false>
 cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc, int* err,
                              cudaStream_t st) {
   using C = cplx_t<T>;
   constexpr int M = 1 << LG, N = 2 * M;
+  const bool dep = BEAM || jb.j[0].rho2.rho2;
   if constexpr (sizeof(T) == 8) {  // double rows: on integers
-    return launch_row_fx<LG, SWEEP, 1, BEAM>(jb, 1, 1, BEAM, twc, err, st);
+    return launch_row_fx<LG, SWEEP, 1, BEAM>(jb, 1, 1, dep, twc, err, st);
   } else if constexpr (row_ldg_shape<T, LG, SWEEP, V>()) {  // float rows of 4096 pixels
     constexpr auto kern = row_fft3_ldg_kernel<1, BEAM>;
     cudaError_t e = ensure_smem_attr<kern>(RowLdgShape::smem);
     if (e) return e;
     const int grid = row_ldg_grid<kern>(1);
     if (grid < 1) return cudaErrorInvalidConfiguration;
-    if constexpr (BEAM)
+    if (dep)
       return launch_dependent(kern, dim3(grid), dim3(RowLdgShape::TT), RowLdgShape::smem, st, jb, twc);
     kern<<<grid, RowLdgShape::TT, RowLdgShape::smem, st>>>(jb, twc);
     return cudaGetLastError();
@@ -72,8 +74,7 @@ cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc,
       if (per_sm < 1) per_sm = 1;
       if (grid > per_sm * current_device_sms()) grid = per_sm * current_device_sms();
     }
-    if constexpr (BEAM)
-      return launch_dependent(kern, dim3(grid), dim3(SH::threads), smem, st, jb, twc, err);
+    if (dep) return launch_dependent(kern, dim3(grid), dim3(SH::threads), smem, st, jb, twc, err);
     kern<<<grid, SH::threads, smem, st>>>(jb, twc, err);
     return cudaGetLastError();
   }
@@ -86,7 +87,7 @@ template <typename T, int N> constexpr bool has_alt_radix() {
 
 template <typename T, int LG, bool SWEEP>
 cudaError_t launch_row3(const T* image, const T* I, const SweepParams& sp, const void* tw,
-                        void* F1, const double* rho2, double S, int* err, const T* beam,
+                        void* F1, const UvExtent& rho2, double S, int* err, const T* beam,
                         cudaStream_t st, int radix, int kc) {
   using C = cplx_t<T>;
   const C* twc = static_cast<const C*>(tw);
@@ -110,7 +111,7 @@ cudaError_t launch_row3(const T* image, const T* I, const SweepParams& sp, const
 }
 
 template <typename T, int LG, int V = FftV<T>::V>
-cudaError_t launch_col3_kern(const void* F1, void* Gw, const void* tw, const double* rho2, double S,
+cudaError_t launch_col3_kern(const void* F1, void* Gw, const void* tw, const UvExtent& rho2, double S,
                              int kc_hint, bool full, bool even, cudaStream_t st) {
   using C = cplx_t<T>;
   constexpr int N = 1 << LG;
@@ -136,7 +137,7 @@ cudaError_t launch_col3_kern(const void* F1, void* Gw, const void* tw, const dou
 }
 
 template <typename T, int LG>
-cudaError_t launch_col3(const void* F1, void* Gw, const void* tw, const double* rho2, double S,
+cudaError_t launch_col3(const void* F1, void* Gw, const void* tw, const UvExtent& rho2, double S,
                         int kc_hint, bool full, bool even, cudaStream_t st, int radix) {
   if constexpr (has_alt_radix<T, (1 << LG)>()) {
     if (radix == kAltRadix)
@@ -147,7 +148,7 @@ cudaError_t launch_col3(const void* F1, void* Gw, const void* tw, const double* 
 
 template <typename T, int LG>
 cudaError_t row3_switch(int lg, const T* image, const T* I, const SweepParams& sp,
-                        const void* tw, void* F1, const double* rho2, double S, int* err,
+                        const void* tw, void* F1, const UvExtent& rho2, double S, int* err,
                         const T* beam, cudaStream_t st, int radix, int kc) {
   if constexpr (LG > 12) {
     return cudaErrorNotSupported;
@@ -165,7 +166,7 @@ cudaError_t row3_switch(int lg, const T* image, const T* I, const SweepParams& s
 template <typename T> constexpr int col3_max_lg() { return max_col_lg<T>(); }
 
 template <typename T, int LG>
-cudaError_t col3_switch(int lg, const void* F1, void* Gw, const void* tw, const double* rho2,
+cudaError_t col3_switch(int lg, const void* F1, void* Gw, const void* tw, const UvExtent& rho2,
                         double S, int kc_hint, bool full, bool even, cudaStream_t st, int radix) {
   if constexpr (LG > col3_max_lg<T>()) {
     return cudaErrorNotSupported;
@@ -183,14 +184,14 @@ inline int ilog2i(int n) {
 
 template <typename T>
 cudaError_t row_fft3(const T* image, const T* I, const SweepParams& sp, int N, const void* tw,
-                     void* F1, const double* rho2, double S, int* err, const T* beam,
+                     void* F1, const UvExtent& rho2, double S, int* err, const T* beam,
                      cudaStream_t st, int radix, int kc) {
   constexpr int LG0 = ilog2c(FftV<T>::V);
   return row3_switch<T, LG0>(ilog2i(N / 2), image, I, sp, tw, F1, rho2, S, err, beam, st, radix, kc);
 }
 
 template <typename T>
-cudaError_t col_fft3(const void* F1, void* Gw, int N, const void* tw, const double* rho2, double S,
+cudaError_t col_fft3(const void* F1, void* Gw, int N, const void* tw, const UvExtent& rho2, double S,
                      int kc_hint, bool full, bool even, cudaStream_t st, int radix) {
   constexpr int LG0 = ilog2c(FftV<T>::V);
   return col3_switch<T, LG0>(ilog2i(N), F1, Gw, tw, rho2, S, kc_hint, full, even, st, radix);

@@ -7,6 +7,8 @@
 
 #include <cmath>
 
+#include "gal_common.cuh"
+
 namespace gal {
 
 // Parameters of the primary-beam tables (Sect. 2.1): c = 4 ln 2 / fwhm^2 and
@@ -45,6 +47,8 @@ struct MultiSources {
   const double* amp;
 };
 
+constexpr size_t kExtentState = 16;  // Launch::extent
+
 // Host launchers, one explicit instantiation per precision.
 template <typename T> struct Launch {
   static cudaError_t init();  // kernel attributes; once per process
@@ -55,7 +59,9 @@ template <typename T> struct Launch {
   static int gather_blocks_per_sm(bool chi2, size_t window_smem);
   // tw: kTwUnits N complex values (TwTab)
   static cudaError_t twiddles(void* tw, int N, cudaStream_t st);
-  static cudaError_t extent(const T* u, const T* v, int64_t M, double* rho2, int blocks,
+  // *out (device or mapped host memory) = max_k u_k^2 + v_k^2; state: kExtentState
+  // bytes, zero at rest, of calls that do not overlap
+  static cudaError_t extent(const T* u, const T* v, int64_t M, double* out, void* state, int sms,
                             cudaStream_t st);
   // u = u_m nu / c, v = v_m nu / c (metres and Hz to wavelengths), in FP64,
   // rounded once to T
@@ -71,7 +77,7 @@ template <typename T> struct Launch {
   // thread of the compile-time FFT stages (kAltRadix, or any other value for FftV);
   // kc_hint: window columns if the host knows them (0: unknown)
   static cudaError_t row_pass(const T* image, const T* I, const SweepParams& sp, int N,
-                              const void* tw, void* F1, const double* rho2, double S, int* err,
+                              const void* tw, void* F1, const UvExtent& rho2, double S, int* err,
                               const T* beam, cudaStream_t st, int radix = 0, int kc_hint = 0);
   // primary-beam tables (2 N values) for a beam of FWHM fwhm > 0 on the
   // pointing centre, seen from a model moved by (dRA, dDec) at position angle PA
@@ -83,10 +89,10 @@ template <typename T> struct Launch {
   // full-plane window of full_cols (lengths of the compile-time passes only);
   // even: F1 comes from a row pass that kept half the rows (even_profile)
   static cudaError_t col_pass(const void* F1, void* Gw, int N, const void* tw,
-                              const double* rho2, double S, int kc_hint, bool full, bool even,
+                              const UvExtent& rho2, double S, int kc_hint, bool full, bool even,
                               cudaStream_t st, int radix = 0);
   // ms: multi-source offsets (null: the single offset of gp)
-  static cudaError_t gather(const void* Gw, const GatherParams& gp, const double* rho2,
+  static cudaError_t gather(const void* Gw, const GatherParams& gp, const UvExtent& rho2,
                             const T* u, const T* v, const T* re, const T* im, const T* w,
                             int64_t M, void* vis, double* partials, unsigned* counter,
                             double* chi2, size_t window_smem, bool edge, int blocks,
@@ -101,10 +107,10 @@ template <typename T> struct Plane {
   static bool supported(int N);  // transform lengths of the full-plane row pass
   // err: bit 2 is set if a staged copy's wait timed out (never expected)
   static cudaError_t rows(const T* image, const T* I, const SweepParams& sp, int N,
-                          const void* tw, void* F1, const double* rho2, double S, const T* beam,
+                          const void* tw, void* F1, const UvExtent& rho2, double S, const T* beam,
                           int* err, cudaStream_t st);
   static int gather_blocks_per_sm(bool chi2, size_t window_smem);
-  static cudaError_t gather(const void* Gw, const GatherParams& gp, const double* rho2,
+  static cudaError_t gather(const void* Gw, const GatherParams& gp, const UvExtent& rho2,
                             const T* u, const T* v, const T* re, const T* im, const T* w,
                             int64_t M, void* vis, double* partials, unsigned* counter,
                             double* chi2, size_t window_smem, bool edge, int blocks,
@@ -147,7 +153,7 @@ struct BatchItem {
   SweepParams sp;
   int N;
   double S;            // N * dxy
-  const double* rho2;  // device: squared uv extent of the observation
+  UvExtent rho2;       // of the observation (host-known)
   int Kc, nrw;         // kept window (same rule as the kernels' bounds)
   void* F1;            // workspace: Kc columns of N complex values
   void* Gw;            // workspace: the window, nrw x Kc complex (+16 B)
@@ -199,10 +205,10 @@ template <typename T> struct BatchLaunch {
 // the length is outside their range (the caller then uses the generic passes).
 template <typename T>
 cudaError_t row_fft3(const T* image, const T* I, const SweepParams& sp, int N, const void* tw,
-                     void* F1, const double* rho2, double S, int* err, const T* beam,
+                     void* F1, const UvExtent& rho2, double S, int* err, const T* beam,
                      cudaStream_t st, int radix, int kc);
 template <typename T>
-cudaError_t col_fft3(const void* F1, void* Gw, int N, const void* tw, const double* rho2, double S,
+cudaError_t col_fft3(const void* F1, void* Gw, int N, const void* tw, const UvExtent& rho2, double S,
                      int kc_hint, bool full, bool even, cudaStream_t st, int radix);
 
 }  // namespace gal

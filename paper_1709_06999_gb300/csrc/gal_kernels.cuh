@@ -66,40 +66,104 @@ __global__ void twiddle_kernel(cplx_t<T>* __restrict__ tw, int N) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// uv extent: *rho2 = max(*rho2, max_k u_k^2 + v_k^2) (NaN points ignored).
-// Non-negative doubles order like their bit patterns, so atomicMax on the
-// 64-bit pattern is an exact maximum.
-// ---------------------------------------------------------------------------
+template <typename T> struct Vec16;
+template <> struct Vec16<float> { using type = float4; static constexpr int W = 4; };
+template <> struct Vec16<double> { using type = double2; static constexpr int W = 2; };
+
 template <typename T>
-__global__ void extent_kernel(const T* __restrict__ u, const T* __restrict__ v, int64_t M,
-                              double* __restrict__ rho2) {
-  double m = 0.0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < M;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const double a = (double)u[k], b = (double)v[k];
-    const double r = a * a + b * b;
-    if (r > m) m = r;
+__device__ __forceinline__ void load16(const T* __restrict__ p, int64_t q, T (&out)[Vec16<T>::W]) {
+  using V = typename Vec16<T>::type;
+  const V x = __ldcs(reinterpret_cast<const V*>(p) + q);
+  if constexpr (Vec16<T>::W == 4) {
+    out[0] = x.x; out[1] = x.y; out[2] = x.z; out[3] = x.w;
+  } else {
+    out[0] = x.x; out[1] = x.y;
   }
+}
+
+// ---------------------------------------------------------------------------
+// uv extent: *out = max_k u_k^2 + v_k^2 over the points (NaN points ignored).
+// Non-negative doubles order like their bit patterns, so integer maxima are
+// exact.  The last block to arrive hands the result over and leaves `state` zero
+// again, so no clearing pass precedes a call.
+//
+// GB300 does FP64 slowly, so a thread screens its float points in float: a point
+// whose float sum of squares is more than 2^-20 above the largest so far replaces
+// it, one more than that below is dropped, and only near ties, and the survivor at
+// the end, are squared and added in FP64.  5e6 points: float 54 -> 17 us, double
+// 35 -> 24 us.
+// ---------------------------------------------------------------------------
+struct ExtentState {
+  unsigned long long top;
+  unsigned count, pad;
+};
+static_assert(sizeof(ExtentState) == kExtentState, "layout");
+
+template <typename T> struct ExtentAcc {
+  unsigned long long top = 0;              // bits of the largest FP64 sum
+  float above = -1.f, below = -1.f;        // float: the survivor's sum, 2^-20 up and down
+  T bu = (T)0, bv = (T)0;                  // the survivor
+  __device__ __forceinline__ void exact(T u, T v) {
+    const double a = (double)u, b = (double)v;
+    const unsigned long long r = (unsigned long long)__double_as_longlong(fma(a, a, b * b));
+    if (r > top && r <= 0x7ff0000000000000ull) top = r;  // NaN lies above infinity
+  }
+  __device__ __forceinline__ void add(T u, T v) {
+    if constexpr (sizeof(T) == 4) {
+      const float s = fmaf(u, u, v * v);
+      if (s > above && s >= 1e-30f) {  // (smaller sums may be denormal in float)
+        above = s * (1.f + 9.5367431640625e-7f);
+        below = s * (1.f - 9.5367431640625e-7f);
+        bu = u;
+        bv = v;
+      } else if (s >= below) {
+        exact(u, v);
+      }
+    } else {
+      exact(u, v);
+    }
+  }
+  __device__ __forceinline__ unsigned long long result() {
+    if constexpr (sizeof(T) == 4) exact(bu, bv);
+    return top;
+  }
+};
+
+constexpr int kExtentThreads = 512;
+template <typename T>
+__global__ void __launch_bounds__(kExtentThreads)
+extent_kernel(const T* __restrict__ u, const T* __restrict__ v, int64_t M, int vec,
+              ExtentState* __restrict__ state, double* __restrict__ out) {
+  grid_dep_launch();  // the row pass may be scheduled meanwhile
+  constexpr int W = Vec16<T>::W;
+  ExtentAcc<T> acc;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t nq = vec ? M / W : 0;
+  for (int64_t q = t0; q < nq; q += stride) {
+    T a[W], b[W];
+    load16(u, q, a);
+    load16(v, q, b);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double x = __shfl_down_sync(0xffffffffu, m, o);
-    if (x > m) m = x;
+    for (int e = 0; e < W; ++e) acc.add(a[e], b[e]);
   }
-  __shared__ double ws[32];
+  for (int64_t k = nq * W + t0; k < M; k += stride) acc.add(u[k], v[k]);
+  unsigned long long m = acc.result();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
+  __shared__ unsigned long long ws[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) ws[warp] = m;
   __syncthreads();
-  if (warp == 0) {
-    m = lane < (int)(blockDim.x >> 5) ? ws[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double x = __shfl_down_sync(0xffffffffu, m, o);
-      if (x > m) m = x;
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = max(m, ws[i]);
+    if (m) atomicMax(&state->top, m);
+    __threadfence();
+    if (atomicAdd(&state->count, 1u) == gridDim.x - 1) {
+      __threadfence();
+      *out = __longlong_as_double((long long)atomicExch(&state->top, 0ull));
+      state->count = 0u;
     }
-    if (lane == 0 && m > 0.0)
-      atomicMax(reinterpret_cast<unsigned long long*>(rho2),
-                (unsigned long long)__double_as_longlong(m));
   }
 }
 
@@ -318,7 +382,7 @@ __device__ __forceinline__ cplx_t<T> beam_pair(cplx_t<T> z, const T* __restrict_
 template <typename T, bool SWEEP>
 __global__ void __launch_bounds__(1024) row_pass_kernel(const T* __restrict__ image, const T* __restrict__ I,
                                 SweepT<T> sp, int N, const cplx_t<T>* __restrict__ tw,
-                                cplx_t<T>* __restrict__ F1, const double* __restrict__ rho2,
+                                cplx_t<T>* __restrict__ F1, const __grid_constant__ UvExtent rho2,
                                 double S, const T* __restrict__ beam) {
   using C = cplx_t<T>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -371,7 +435,7 @@ __global__ void __launch_bounds__(1024) row_pass_kernel(const T* __restrict__ im
 template <typename T>
 __global__ void __launch_bounds__(1024)
 col_pass_kernel(const cplx_t<T>* __restrict__ F1, cplx_t<T>* __restrict__ Gp, int N,
-                const cplx_t<T>* __restrict__ tw, const double* __restrict__ rho2, double S) {
+                const cplx_t<T>* __restrict__ tw, const __grid_constant__ UvExtent rho2, double S) {
   using C = cplx_t<T>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C* sm = reinterpret_cast<C*>(smem_raw);
@@ -486,7 +550,7 @@ row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>
   const T* __restrict__ I = jb.I;
   const SweepT<T>& sp = jb.sp;
   C* __restrict__ F1 = jb.F1;
-  const double* __restrict__ rho2 = jb.rho2;
+  const UvExtent& rho2 = jb.rho2;
   const double S = jb.S;
   const T* __restrict__ beam = BEAM ? jb.beam : nullptr;
   constexpr int M = 1 << LG, N = 2 * M;
@@ -828,7 +892,7 @@ col_fft3_kernel(const __grid_constant__ Jobs<ColJob<T>, K> jobs, const cplx_t<T>
   const ColJob<T>& jb = jobs.j[K == 1 ? 0 : blockIdx.y];
   const cplx_t<T>* __restrict__ F1 = jb.F1;
   cplx_t<T>* __restrict__ Gw = jb.Gw;
-  const double* __restrict__ rho2 = jb.rho2;
+  const UvExtent& rho2 = jb.rho2;
   const double S = jb.S;
   grid_dep_launch();  // the gather may start its prologue on the SMs we leave idle
   using C = cplx_t<T>;
@@ -979,14 +1043,14 @@ template <typename T> struct RowJob {
   const T* I;           // profile (SWEEP)
   SweepT<T> sp;
   cplx_t<T>* F1;        // row-pass output, column-major (Kc columns of N)
-  const double* rho2;   // squared uv extent of the request's points
+  UvExtent rho2;        // of the request's points
   double S;             // nxy * dxy
   const T* beam;        // primary-beam factors (beam_table_kernel), null: none
 };
 template <typename T> struct ColJob {
   const cplx_t<T>* F1;
   cplx_t<T>* Gw;        // window output, nrw x Kc (full plane: nrw x W)
-  const double* rho2;
+  UvExtent rho2;
   double S;
   int full;             // 1: the full-plane window (full_cols(bd, N).W columns)
   int even;             // 1: F1 holds rows 0 .. N/2 only, row N - i being row i
@@ -1014,7 +1078,7 @@ template <> struct GatherT<double> {
 template <typename T> struct GatherJob {
   const cplx_t<T>* Gw;
   GatherT<T> p;
-  const double* rho2;
+  UvExtent rho2;
   const T *u, *v, *re, *im, *w;
   int64_t M;
   int vec;              // all point arrays 16-byte aligned
@@ -1563,21 +1627,6 @@ template <typename T> struct Acc;
 template <> struct Acc<float> { using type = AccF; };
 template <> struct Acc<double> { using type = AccD; };
 
-template <typename T> struct Vec16;
-template <> struct Vec16<float> { using type = float4; static constexpr int W = 4; };
-template <> struct Vec16<double> { using type = double2; static constexpr int W = 2; };
-
-template <typename T>
-__device__ __forceinline__ void load16(const T* __restrict__ p, int64_t q, T (&out)[Vec16<T>::W]) {
-  using V = typename Vec16<T>::type;
-  const V x = __ldcs(reinterpret_cast<const V*>(p) + q);
-  if constexpr (Vec16<T>::W == 4) {
-    out[0] = x.x; out[1] = x.y; out[2] = x.z; out[3] = x.w;
-  } else {
-    out[0] = x.x; out[1] = x.y;
-  }
-}
-
 __device__ __forceinline__ double block_sum(double x, double* ws) {
   // (a warp of zeros has nothing to add: idle warps stay off the FP64 pipe)
   if (__any_sync(0xffffffffu, (__double_as_longlong(x) << 1) != 0)) {
@@ -1745,7 +1794,7 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
   const GatherJob<T>& jb = jobs.j[K == 1 ? 0 : blockIdx.y];
   const C* __restrict__ Gw = jb.Gw;
   const GatherT<T>& p = jb.p;
-  const double* __restrict__ rho2 = jb.rho2;
+  const UvExtent& rho2 = jb.rho2;
   const T* __restrict__ u = jb.u;
   const T* __restrict__ v = jb.v;
   const T* __restrict__ re = jb.re;
@@ -2028,14 +2077,13 @@ template <typename T> cudaError_t Launch<T>::twiddles(void* tw, int N, cudaStrea
 }
 
 template <typename T>
-cudaError_t Launch<T>::extent(const T* u, const T* v, int64_t M, double* rho2, int blocks,
+cudaError_t Launch<T>::extent(const T* u, const T* v, int64_t M, double* out, void* state, int sms,
                               cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(rho2, 0, sizeof(double), st);
-  if (e) return e;
-  if (M <= 0) return cudaSuccess;
-  const int64_t need = (M + 255) / 256;
-  const int grid = (int)(need < blocks ? need : blocks);
-  extent_kernel<T><<<grid, 256, 0, st>>>(u, v, M, rho2);
+  const int vec = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15u) == 0;
+  const int64_t need = ((vec ? M / Vec16<T>::W : M) + kExtentThreads - 1) / kExtentThreads;
+  const int64_t cap = 2 * (int64_t)sms;  // two blocks an SM: enough loads in flight, few arrivals
+  const int grid = (int)(need < 1 ? 1 : need < cap ? need : cap);
+  extent_kernel<T><<<grid, kExtentThreads, 0, st>>>(u, v, M, vec, static_cast<ExtentState*>(state), out);
   return cudaGetLastError();
 }
 
@@ -2074,7 +2122,7 @@ cudaError_t Launch<T>::sweep(const T* I, const SweepParams& sp, int N, T* img, i
 
 template <typename T>
 cudaError_t Launch<T>::row_pass(const T* image, const T* I, const SweepParams& sp, int N,
-                                const void* tw, void* F1, const double* rho2, double S, int* err,
+                                const void* tw, void* F1, const UvExtent& rho2, double S, int* err,
                                 const T* beam, cudaStream_t st, int radix, int kc_hint) {
   using C = cplx_t<T>;
   const int M = N / 2;
@@ -2118,7 +2166,7 @@ bool Launch<T>::even_profile(int N) {
 
 template <typename T>
 cudaError_t Launch<T>::col_pass(const void* F1, void* Gw, int N, const void* tw,
-                                const double* rho2, double S, int kc_hint, bool full, bool even,
+                                const UvExtent& rho2, double S, int kc_hint, bool full, bool even,
                                 cudaStream_t st, int radix) {
   using C = cplx_t<T>;
   if (N >= FftV<T>::V) {
@@ -2142,7 +2190,7 @@ cudaError_t Launch<T>::col_pass(const void* F1, void* Gw, int N, const void* tw,
 }
 
 template <typename T>
-cudaError_t Launch<T>::gather(const void* Gw, const GatherParams& gp, const double* rho2,
+cudaError_t Launch<T>::gather(const void* Gw, const GatherParams& gp, const UvExtent& rho2,
                               const T* u, const T* v, const T* re, const T* im, const T* w,
                               int64_t M, void* vis, double* partials, unsigned* counter,
                               double* chi2, size_t window_smem, bool edge, int blocks,

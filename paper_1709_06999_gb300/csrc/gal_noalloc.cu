@@ -43,7 +43,7 @@ constexpr int kMaxDevices = 64;
 struct DeviceSetup {
   unsigned char* base = nullptr;  // device address of g_noalloc_scratch
   int gather_blocks = 0;
-  int aux_blocks = 0;
+  int sms = 0;
 };
 DeviceSetup g_setup[kMaxDevices];
 std::mutex g_setup_mutex;
@@ -64,7 +64,7 @@ int setup_current_device(DeviceSetup** out) {
       return GAL_E_DEVICE;
     int blocks = sms * gal::Launch<float>::gather_blocks_per_sm(true, 0);
     s.gather_blocks = blocks < kMaxBlocks ? blocks : kMaxBlocks;
-    s.aux_blocks = sms * 8;
+    s.sms = sms;
     s.base = static_cast<unsigned char*>(p);
   }
   *out = &s;
@@ -111,22 +111,25 @@ extern "C" int gal_chi2_image_noalloc_f32(const float* image, int nxy, double dx
   int* err = reinterpret_cast<int*>(s->base + kOffErr);
 
   // The array keeps whatever the previous call left: reset what must start at
-  // zero (the extent launcher clears rho2 itself), rebuild the twiddles for
+  // zero (the extent pass writes rho2), rebuild the twiddles for
   // this nxy.
   if (cudaMemsetAsync(counter, 0, sizeof(unsigned), cs) != cudaSuccess) return GAL_E_CUDA;
   if (cudaMemsetAsync(err, 0, sizeof(int), cs) != cudaSuccess) return GAL_E_CUDA;
   if (gal::Launch<float>::twiddles(tw, nxy, cs) != cudaSuccess) return GAL_E_CUDA;
-  if (gal::Launch<float>::extent(u, v, M, rho2, s->aux_blocks, cs) != cudaSuccess)
+  void* ext_state = s->base + kOffRho2 + 128;
+  if (cudaMemsetAsync(ext_state, 0, gal::kExtentState, cs) != cudaSuccess) return GAL_E_CUDA;
+  if (gal::Launch<float>::extent(u, v, M, rho2, ext_state, s->sms, cs) != cudaSuccess)
     return GAL_E_CUDA;
+  const gal::UvExtent ext{rho2, gal::Bounds{}};
   const double S = (double)nxy * dxy;
   gal::SweepParams none{};
   int dev = 0, rv = 0, cv = 0;
   cudaGetDevice(&dev);
   gal::fft_plan_lookup_f32(dev, nxy, &rv, &cv);
-  if (gal::Launch<float>::row_pass(image, nullptr, none, nxy, tw, F1, rho2, S, err, nullptr, cs,
+  if (gal::Launch<float>::row_pass(image, nullptr, none, nxy, tw, F1, ext, S, err, nullptr, cs,
                                    rv) != cudaSuccess)
     return GAL_E_CUDA;
-  if (gal::Launch<float>::col_pass(F1, Gw, nxy, tw, rho2, S, 0, false, false, cs, cv) != cudaSuccess)
+  if (gal::Launch<float>::col_pass(F1, Gw, nxy, tw, ext, S, 0, false, false, cs, cv) != cudaSuccess)
     return GAL_E_CUDA;
   gal::GatherParams gp;
   gp.cpa = std::cos(PA);
@@ -135,7 +138,7 @@ extern "C" int gal_chi2_image_noalloc_f32(const float* image, int nxy, double dx
   gp.phx = dRA;
   gp.phy = dDec;
   gp.N = nxy;
-  if (gal::Launch<float>::gather(Gw, gp, rho2, u, v, re, im, w, M, nullptr, partials, counter,
+  if (gal::Launch<float>::gather(Gw, gp, ext, u, v, re, im, w, M, nullptr, partials, counter,
                                  chi2_out, 0, true, s->gather_blocks, nullptr, cs) != cudaSuccess)
     return GAL_E_CUDA;
   noalloc_status_kernel<<<1, 1, 0, cs>>>(err, chi2_out);

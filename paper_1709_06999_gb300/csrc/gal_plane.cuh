@@ -292,7 +292,7 @@ template <typename T> bool Plane<T>::supported(int N) {
 
 template <typename T>
 cudaError_t Plane<T>::rows(const T* image, const T* I, const SweepParams& sp, int N,
-                           const void* tw, void* F1, const double* rho2, double S, const T* beam,
+                           const void* tw, void* F1, const UvExtent& rho2, double S, const T* beam,
                            int* err, cudaStream_t st) {
   if (!supported(N)) return cudaErrorNotSupported;
   RowJob<T> jb{image, I, I ? sweep_cast<T>(sp) : SweepT<T>{}, static_cast<cplx_t<T>*>(F1), rho2, S,
@@ -329,7 +329,7 @@ template <typename T> int Plane<T>::gather_blocks_per_sm(bool chi2, size_t windo
 }
 
 template <typename T>
-cudaError_t Plane<T>::gather(const void* Gw, const GatherParams& gp, const double* rho2,
+cudaError_t Plane<T>::gather(const void* Gw, const GatherParams& gp, const UvExtent& rho2,
                              const T* u, const T* v, const T* re, const T* im, const T* w,
                              int64_t M, void* vis, double* partials, unsigned* counter,
                              double* chi2, size_t window_smem, bool edge, int blocks,

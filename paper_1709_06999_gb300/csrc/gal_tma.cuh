@@ -69,11 +69,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 
 // Programmatic dependent launch (sm_90 and later).  A kernel launched with
 // programmatic stream serialization may start before the preceding kernel in
-// its stream has finished; grid_dep_wait() blocks until that kernel has
+// its stream has finished; grid_dep_wait() (gal_common.cuh) blocks until that kernel has
 // completed and its memory operations are visible (a no-op when the kernel
 // was launched normally).  grid_dep_launch() lets the next kernel, if it was
 // launched that way, begin launching; it changes nothing else.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
 
 // bring the line holding p into L2 (no register result)
