@@ -1562,10 +1562,19 @@ __device__ __forceinline__ double2 sample_point(const cplx_t<double>* __restrict
   return bad ? make_double2(fx_nan(), fx_nan()) : out;
 }
 
-// per-thread compensated accumulators
-// block-wide sum of one double per thread, fixed order; result valid in thread 0
-__device__ __forceinline__ double block_sum(double x, double* ws);
+// Sum of one double per lane, fixed order, valid in lane 0.  (A warp of zeros has
+// nothing to add: idle warps stay off the FP64 pipe.)
+__device__ __forceinline__ double warp_sum(double x) {
+  if (__any_sync(0xffffffffu, (__double_as_longlong(x) << 1) != 0)) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+  }
+  return x;
+}
 
+// per-thread compensated accumulators.  A block's total is formed in two steps:
+// put() leaves each warp's total in a slot of 32 doubles, and after a barrier one
+// warp's cross() adds a slot's entries (valid in lane 0).
 struct AccF {  // Kahan: s holds the sum, c the negated lost low-order part
   float s = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float x) {
@@ -1574,40 +1583,38 @@ struct AccF {  // Kahan: s holds the sum, c the negated lost low-order part
     c = (t - s) - y;
     s = t;
   }
-  // Block total (valid in thread 0): a float-float tree inside each warp and
-  // across the warps, converted to FP64 once.  GB300 issues FP64 at a small
-  // fraction of the FP32 rate, and a dependent FP64 tree across 16 warps
-  // added about 1 us to the end of every block; the float-float sums carry
-  // about 48 significant bits.  The sum over blocks stays FP64.
-  __device__ __forceinline__ double block_total(double* ws) const {
-    auto warp_tree = [](ff a) {
+  // A float-float tree inside each warp and across the warps, converted to FP64
+  // once.  GB300 issues FP64 at a small fraction of the FP32 rate, and a
+  // dependent FP64 tree across 16 warps added about 1 us to the end of every
+  // block; the float-float sums carry about 48 significant bits.  The sum over
+  // blocks stays FP64.
+  static __device__ __forceinline__ ff warp_tree(ff a) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        ff b;
-        b.hi = __shfl_down_sync(0xffffffffu, a.hi, o);
-        b.lo = __shfl_down_sync(0xffffffffu, a.lo, o);
-        a = ff_add(a, b);
-      }
-      return a;
-    };
+    for (int o = 16; o > 0; o >>= 1) {
+      ff b;
+      b.hi = __shfl_down_sync(0xffffffffu, a.hi, o);
+      b.lo = __shfl_down_sync(0xffffffffu, a.lo, o);
+      a = ff_add(a, b);
+    }
+    return a;
+  }
+  __device__ __forceinline__ void put(double* slot) const {
     ff a;
     a.hi = s;
     a.lo = -c;
     a = warp_tree(a);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float2* wf = reinterpret_cast<float2*>(ws);  // 32 doubles hold 32 float pairs
-    __syncthreads();
-    if (lane == 0) wf[warp] = make_float2(a.hi, a.lo);
-    __syncthreads();
-    double x = 0.0;
-    if (warp == 0) {
-      const float2 w = lane < (int)(blockDim.x >> 5) ? wf[lane] : make_float2(0.f, 0.f);
-      a.hi = w.x;
-      a.lo = w.y;
-      a = warp_tree(a);
-      x = (double)a.hi + (double)a.lo;
-    }
-    return x;
+    if ((threadIdx.x & 31) == 0)
+      reinterpret_cast<float2*>(slot)[threadIdx.x >> 5] = make_float2(a.hi, a.lo);
+  }
+  static __device__ __forceinline__ double cross(const double* slot) {
+    const int lane = threadIdx.x & 31;
+    const float2 w = lane < (int)(blockDim.x >> 5) ? reinterpret_cast<const float2*>(slot)[lane]
+                                                   : make_float2(0.f, 0.f);
+    ff a;
+    a.hi = w.x;
+    a.lo = w.y;
+    a = warp_tree(a);
+    return (double)a.hi + (double)a.lo;
   }
 };
 struct AccD {  // Neumaier
@@ -1621,29 +1628,26 @@ struct AccD {  // Neumaier
     s = t;
   }
   __device__ __forceinline__ double value() const { return s + c; }
-  __device__ __forceinline__ double block_total(double* ws) const { return block_sum(value(), ws); }
+  __device__ __forceinline__ void put(double* slot) const {
+    const double x = warp_sum(value());
+    if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = x;
+  }
+  static __device__ __forceinline__ double cross(const double* slot) {
+    const int lane = threadIdx.x & 31;
+    return warp_sum(lane < (int)(blockDim.x >> 5) ? slot[lane] : 0.0);
+  }
 };
 template <typename T> struct Acc;
 template <> struct Acc<float> { using type = AccF; };
 template <> struct Acc<double> { using type = AccD; };
 
+// block-wide sum of one double per thread, fixed order; result valid in thread 0
 __device__ __forceinline__ double block_sum(double x, double* ws) {
-  // (a warp of zeros has nothing to add: idle warps stay off the FP64 pipe)
-  if (__any_sync(0xffffffffu, (__double_as_longlong(x) << 1) != 0)) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  x = warp_sum(x);
   __syncthreads();
-  if (lane == 0) ws[warp] = x;
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = x;
   __syncthreads();
-  x = 0.0;
-  if (warp == 0) {
-    x = lane < (int)(blockDim.x >> 5) ? ws[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-  }
-  return x;
+  return threadIdx.x < 32 ? AccD::cross(ws) : 0.0;
 }
 
 // SMEM: the block first copies the kept window (nrw x Kc nodes) into shared
@@ -1674,15 +1678,18 @@ template <typename T, bool CHI2> struct PointGroup {
 // Grid-stride layout of the vector groups: whole rounds of gstride groups,
 // then the remainder in equal contiguous slices, one per block (coalesced,
 // and no few blocks run a round more than the rest).
-// nblk blocks, this thread in block bid.
+// nblk blocks; at(bid): this thread in block bid (the divisions are done once,
+// 64-bit ones cost about as much as a point).
 struct GroupSplit {
   int64_t nq, gstride, rounds, slice, rem_q, gtid;
-  __device__ __forceinline__ GroupSplit(int64_t M, int W, int vec, int nblk, int bid) {
+  __device__ __forceinline__ GroupSplit(int64_t M, int W, int vec, int nblk) {
     nq = vec ? M / W : 0;
     gstride = (int64_t)nblk * blockDim.x;
     rounds = nq / gstride;
     const int64_t rem = nq - rounds * gstride;
     slice = (rem + nblk - 1) / nblk;  // <= blockDim.x
+  }
+  __device__ __forceinline__ void at(int bid) {
     rem_q = rounds * gstride + (int64_t)bid * slice + threadIdx.x;
     gtid = (int64_t)bid * blockDim.x + threadIdx.x;
   }
@@ -1824,7 +1831,8 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
   // 256 image with 1e4 points, but the selected address made 4096 / 5e6 3 % slower.)
   // (Single calls only: batched launches are not dependents.)
   constexpr int W = Vec16<T>::W;
-  const GroupSplit gs(M, W, vec, nvb, blockIdx.x);
+  GroupSplit gs(M, W, vec, nvb);
+  gs.at(blockIdx.x);
   PointGroup<T, CHI2> g0;
   const bool pre = K == 1 && gs.rounds > 0;  // uniform over the grid
   if constexpr (K == 1) {
@@ -1876,34 +1884,58 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
       }
     }
   }
-  __shared__ double ws[32];
-  auto run = [&](int vb, const GroupSplit& sp, const PointGroup<T, CHI2>* g0p) {
-    typename Acc<T>::type acc;
+  using ACC = typename Acc<T>::type;
+  auto run = [&](const PointGroup<T, CHI2>* g0p, double* slot) {  // the block gs is at
+    ACC acc;
     if constexpr (SMEM) {
       if (win_ok) {
         gather_points<T, CHI2, true, EDGE, MULTI, FULL>(sw, win, p, u, v, re, im, w, M, vec, vis,
-                                                        acc, mp, g0p, sp, tab);
+                                                        acc, mp, g0p, gs, tab);
       } else {
         const T nan = std::numeric_limits<T>::quiet_NaN();
         if constexpr (CHI2) {
           acc.add(nan);
         } else {
-          for (int64_t k = sp.gtid; k < M; k += sp.gstride) vis[k] = mkc(nan, nan);
+          for (int64_t k = gs.gtid; k < M; k += gs.gstride) vis[k] = mkc(nan, nan);
         }
       }
     } else {
       gather_points<T, CHI2, false, EDGE, MULTI, FULL>(Gw, win, p, u, v, re, im, w, M, vec, vis,
-                                                       acc, mp, g0p, sp, tab);
+                                                       acc, mp, g0p, gs, tab);
     }
-    if constexpr (CHI2) {
-      const double bs = acc.block_total(ws);
-      if (threadIdx.x == 0) partials[vb] = bs;
-    }
+    if constexpr (CHI2) acc.put(slot);
   };
+  // The warps of a batched block run through its virtual blocks without waiting
+  // for one another: each virtual block has its slot, and one barrier at the end
+  // precedes the sums over warps, which the warps share out (two barriers and
+  // three 64-bit divisions to each virtual block before: 64 walkers 1024 / 1e6
+  // 624 -> 573 us, 64 cube channels 379 -> 369 us).
+  constexpr int kSlots = K == 1 ? 1 : kMaxGatherFold;
+  __shared__ double red[kSlots][32];
   if constexpr (K == 1) {
-    run(blockIdx.x, gs, pre ? &g0 : nullptr);
+    run(pre ? &g0 : nullptr, red[0]);
+    if constexpr (CHI2) {
+      __syncthreads();
+      if (threadIdx.x < 32) {
+        const double x = ACC::cross(red[0]);
+        if (threadIdx.x == 0) partials[blockIdx.x] = x;
+      }
+    }
   } else {
-    for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) run(vb, GroupSplit(M, W, vec, nvb, vb), nullptr);
+    for (int vb = blockIdx.x; vb < nvb;) {
+      int n = 0, next = vb;
+      for (; n < kSlots && next < nvb; ++n, next += gridDim.x) {
+        gs.at(next);
+        run(nullptr, red[n]);
+      }
+      __syncthreads();
+      for (int k = threadIdx.x >> 5; k < n; k += (int)(blockDim.x >> 5)) {
+        const double x = ACC::cross(red[k]);
+        if ((threadIdx.x & 31) == 0) partials[vb + k * (int)gridDim.x] = x;
+      }
+      __syncthreads();
+      vb = next;
+    }
   }
   if constexpr (CHI2) {
     __shared__ bool last;
@@ -1925,7 +1957,7 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
         for (int b = threadIdx.x; b < nvb; b += blockDim.x) a.add(__ldcg(partials + b));
         x = a.value();
       }
-      const double tot = block_sum(x, ws);
+      const double tot = block_sum(x, red[0]);
       if (threadIdx.x == 0) {
         *chi2_out = tot;
         *counter = 0u;
