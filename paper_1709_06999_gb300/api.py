@@ -18,6 +18,13 @@ from . import _native
 
 _SUFFIX = {torch.float32: "f32", torch.float64: "f64"}
 
+# The current device and its current stream's handle, without the checks and the
+# Stream object of torch.cuda's functions (about 2 us a call); a Context has
+# initialised CUDA.  Absent in a torch without them: the public functions.
+_current_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream",
+                      lambda d: torch.cuda.current_stream(d).cuda_stream)
+
 
 class GalError(RuntimeError):
     pass
@@ -175,7 +182,7 @@ class Observation:
         if z_order and nu is not None:
             raise ValueError("z_order applies to observations in wavelengths")
         arrays = (u, v, re, im, w) if nu is None else (u, v, nu, re, im, w)
-        tensors = [ctx._dev(t).contiguous() for t in arrays]
+        tensors = [ctx._dev(t) for t in arrays]
         m = tensors[0].numel()
         if any(t.numel() != m for t in tensors):
             raise ValueError("u, v, re, im, w (and nu) must have the same length")
@@ -214,6 +221,8 @@ class Context:
         h = ct.c_void_p()
         _check(None, self.lib.gal_create(ct.byref(h), device))
         self.handle = h
+        self._fns = {}  # entry points by (name, dtype)
+        torch.cuda.init()
 
     # -- plumbing -----------------------------------------------------------
     def close(self):
@@ -229,17 +238,29 @@ class Context:
 
     def _stream(self) -> int:
         # the library enqueues on the calling thread's current device
-        if torch.cuda.current_device() != self.device.index:
-            raise GalError(f"current CUDA device is {torch.cuda.current_device()}, the context's "
-                           f"is {self.device.index}: select it first (torch.cuda.set_device)")
-        return torch.cuda.current_stream(self.device).cuda_stream
+        d = _current_device()
+        if d != self.device.index:
+            raise GalError(f"current CUDA device is {d}, the context's is {self.device.index}: "
+                           "select it first (torch.cuda.set_device)")
+        return _raw_stream(d)
 
     def _dev(self, t):
         if not isinstance(t, torch.Tensor):
             raise TypeError("expected a torch.Tensor")
         if t.device != self.device:
             raise ValueError(f"tensor on {t.device}, context on {self.device}")
-        return t.contiguous()
+        return t if t.is_contiguous() else t.contiguous()
+
+    def _fn(self, name: str, *tensors):
+        """Entry point `name` in the precision the tensors share."""
+        key = (name, tensors[0].dtype)
+        fn = self._fns.get(key)
+        if fn is None:
+            fn = self._fns[key] = getattr(self.lib, f"{name}_{_suffix(tensors[0])}")
+        for t in tensors[1:]:
+            if t.dtype != key[1]:
+                raise TypeError("all arrays of one call must share a dtype")
+        return fn
 
     def workspace_bytes(self) -> int:
         """Device workspace this context holds now (gal_workspace_bytes)."""
@@ -288,10 +309,9 @@ class Context:
     def sweep(self, intensity, Rmin: float, dR: float, nxy: int, dxy: float, inc: float = 0.0,
               out=None):
         I = self._dev(intensity)
-        sfx = _suffix(I)
+        fn = self._fn("gal_sweep", I)
         if out is None:
             out = torch.empty((nxy, nxy), dtype=I.dtype, device=self.device)
-        fn = getattr(self.lib, f"gal_sweep_{sfx}")
         _check(self.handle, fn(self.handle, I.data_ptr(), I.numel(), Rmin, dR, nxy, dxy, inc,
                                out.data_ptr(), self._stream()))
         return out
@@ -302,54 +322,53 @@ class Context:
         primary beam of that FWHM (radians); full_plane uses the
         complex-to-complex spectrum (gal_opts)."""
         img, u, v = self._dev(image), self._dev(u), self._dev(v)
-        sfx = _suffix(img, u, v)
+        opts = _opts(pb_fwhm, full_plane)
+        fn = self._fn("gal_sample_image" if opts is None else "gal_sample_image_ex", img, u, v)
         nxy = img.shape[0]
         if img.dim() != 2 or img.shape[1] != nxy:
             raise ValueError("image must be square")
         m = u.numel()
         if out is None:
             out = torch.empty((m, 2), dtype=img.dtype, device=self.device)
-        opts = _opts(pb_fwhm, full_plane)
         head = (self.handle, img.data_ptr(), nxy, dxy, dRA, dDec, PA)
         tail = (m, u.data_ptr(), v.data_ptr(), out.data_ptr(), self._stream())
         if opts is None:
-            _check(self.handle, getattr(self.lib, f"gal_sample_image_{sfx}")(*head, *tail))
+            _check(self.handle, fn(*head, *tail))
         else:
-            _check(self.handle, getattr(self.lib, f"gal_sample_image_ex_{sfx}")(*head, opts, *tail))
+            _check(self.handle, fn(*head, opts, *tail))
         return out
 
     def sample_profile(self, intensity, Rmin: float, dR: float, nxy: int, dxy: float, u, v,
                        inc: float = 0.0, dRA: float = 0.0, dDec: float = 0.0, PA: float = 0.0,
                        out=None, *, pb_fwhm: float = 0.0, full_plane: bool = False):
         I, u, v = self._dev(intensity), self._dev(u), self._dev(v)
-        sfx = _suffix(I, u, v)
+        opts = _opts(pb_fwhm, full_plane)
+        fn = self._fn("gal_sample_profile" if opts is None else "gal_sample_profile_ex", I, u, v)
         m = u.numel()
         if out is None:
             out = torch.empty((m, 2), dtype=I.dtype, device=self.device)
-        opts = _opts(pb_fwhm, full_plane)
         head = (self.handle, I.data_ptr(), I.numel(), Rmin, dR, nxy, dxy, inc, dRA, dDec, PA)
         tail = (m, u.data_ptr(), v.data_ptr(), out.data_ptr(), self._stream())
         if opts is None:
-            _check(self.handle, getattr(self.lib, f"gal_sample_profile_{sfx}")(*head, *tail))
+            _check(self.handle, fn(*head, *tail))
         else:
-            _check(self.handle,
-                   getattr(self.lib, f"gal_sample_profile_ex_{sfx}")(*head, opts, *tail))
+            _check(self.handle, fn(*head, opts, *tail))
         return out
 
     def chi2_image(self, image, dxy: float, obs: Observation, dRA: float = 0.0, dDec: float = 0.0,
                    PA: float = 0.0, out=None, *, pb_fwhm: float = 0.0, full_plane: bool = False):
         """chi2 as a one-element float64 device tensor (stream-ordered, no sync)."""
         img = self._dev(image)
-        sfx = _suffix(img)
+        opts = _opts(pb_fwhm, full_plane)
+        fn = self._fn("gal_chi2_image" if opts is None else "gal_chi2_image_ex", img)
         if out is None:
             out = torch.empty((), dtype=torch.float64, device=self.device)
-        opts = _opts(pb_fwhm, full_plane)
         head = (self.handle, img.data_ptr(), img.shape[0], dxy, dRA, dDec, PA)
         tail = (obs.handle, out.data_ptr(), self._stream())
         if opts is None:
-            _check(self.handle, getattr(self.lib, f"gal_chi2_image_{sfx}")(*head, *tail))
+            _check(self.handle, fn(*head, *tail))
         else:
-            _check(self.handle, getattr(self.lib, f"gal_chi2_image_ex_{sfx}")(*head, opts, *tail))
+            _check(self.handle, fn(*head, opts, *tail))
         return out
 
     def chi2_profile(self, intensity, Rmin: float, dR: float, nxy: int, dxy: float,
@@ -357,17 +376,16 @@ class Context:
                      PA: float = 0.0, out=None, *, pb_fwhm: float = 0.0,
                      full_plane: bool = False):
         I = self._dev(intensity)
-        sfx = _suffix(I)
+        opts = _opts(pb_fwhm, full_plane)
+        fn = self._fn("gal_chi2_profile" if opts is None else "gal_chi2_profile_ex", I)
         if out is None:
             out = torch.empty((), dtype=torch.float64, device=self.device)
-        opts = _opts(pb_fwhm, full_plane)
         head = (self.handle, I.data_ptr(), I.numel(), Rmin, dR, nxy, dxy, inc, dRA, dDec, PA)
         tail = (obs.handle, out.data_ptr(), self._stream())
         if opts is None:
-            _check(self.handle, getattr(self.lib, f"gal_chi2_profile_{sfx}")(*head, *tail))
+            _check(self.handle, fn(*head, *tail))
         else:
-            _check(self.handle,
-                   getattr(self.lib, f"gal_chi2_profile_ex_{sfx}")(*head, opts, *tail))
+            _check(self.handle, fn(*head, opts, *tail))
         return out
 
     def chi2_image_host_async(self, image_host, dxy: float, obs: Observation, out, index: int = 0,
@@ -417,12 +435,11 @@ class Context:
         """Visibilities of K copies of `image`, copy k scaled by amp[k] and
         shifted by (dRA[k], dDec[k]), all rotated by PA: one FFT for all."""
         img, u, v = self._dev(image), self._dev(u), self._dev(v)
-        sfx = _suffix(img, u, v)
+        fn = self._fn("gal_sample_image_multi", img, u, v)
         K, a, b, c = self._sources(dRA, dDec, amp)
         m = u.numel()
         if out is None:
             out = torch.empty((m, 2), dtype=img.dtype, device=self.device)
-        fn = getattr(self.lib, f"gal_sample_image_multi_{sfx}")
         _check(self.handle, fn(self.handle, img.data_ptr(), img.shape[0], dxy, PA, K, a, b, c, m,
                                u.data_ptr(), v.data_ptr(), out.data_ptr(), self._stream()))
         return out
@@ -430,11 +447,10 @@ class Context:
     def chi2_image_multi(self, image, dxy: float, obs: Observation, dRA, dDec, amp=None,
                          PA: float = 0.0, out=None):
         img = self._dev(image)
-        sfx = _suffix(img)
+        fn = self._fn("gal_chi2_image_multi", img)
         K, a, b, c = self._sources(dRA, dDec, amp)
         if out is None:
             out = torch.empty((), dtype=torch.float64, device=self.device)
-        fn = getattr(self.lib, f"gal_chi2_image_multi_{sfx}")
         _check(self.handle, fn(self.handle, img.data_ptr(), img.shape[0], dxy, PA, K, a, b, c,
                                obs.handle, out.data_ptr(), self._stream()))
         return out
@@ -443,11 +459,10 @@ class Context:
                            obs: Observation, dRA, dDec, amp=None, inc: float = 0.0,
                            PA: float = 0.0, out=None):
         I = self._dev(intensity)
-        sfx = _suffix(I)
+        fn = self._fn("gal_chi2_profile_multi", I)
         K, a, b, c = self._sources(dRA, dDec, amp)
         if out is None:
             out = torch.empty((), dtype=torch.float64, device=self.device)
-        fn = getattr(self.lib, f"gal_chi2_profile_multi_{sfx}")
         _check(self.handle, fn(self.handle, I.data_ptr(), I.numel(), Rmin, dR, nxy, dxy, inc, PA,
                                K, a, b, c, obs.handle, out.data_ptr(), self._stream()))
         return out

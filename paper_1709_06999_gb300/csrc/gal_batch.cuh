@@ -52,17 +52,13 @@ cudaError_t rows(const BatchItem* it, const int* idx, int n, const void* tw, int
     if (e) return e;
     int x = row_ldg_grid<kern>(n) * (sh.row_blocks < 1 ? 1 : sh.row_blocks);
     if (x > RowLdgShape::N) x = RowLdgShape::N;
-    if (x < 1) return cudaErrorInvalidConfiguration;
     kern<<<dim3(x, n), RowLdgShape::TT, RowLdgShape::smem, st>>>(jb, twc);
   } else if constexpr (!SWEEP) {
     constexpr auto kern = row_fft3_kernel<T, LG, true, false, kBatchJobs, BEAM, row_min_threads(PAIRS), 2, V>;
     const size_t smem = 128 + (size_t)3 * SH::G * SH::RS * sizeof(C);
     cudaError_t e = ensure_smem_attr<kern>(smem);
     if (e) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SH::threads, smem);
-    if (e) return e;
-    if (per_sm < 1) per_sm = 1;
+    const int per_sm = resident_blocks<kern>(SH::threads, smem);
     // persistent blocks per request: the GPU's resident blocks (times the
     // shape's factor) shared by the chunk's requests
     int x = (per_sm * current_device_sms() * (sh.row_blocks < 1 ? 1 : sh.row_blocks) + n - 1) / n;

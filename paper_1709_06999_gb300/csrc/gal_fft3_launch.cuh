@@ -17,12 +17,8 @@ template <typename T, int LG, bool SWEEP, int V> constexpr bool row_ldg_shape() 
 // its persistent grid: the resident blocks of the device, shared by the
 // `n` requests of a launch (grid row y = request), at most one row each
 template <auto Kern> int row_ldg_grid(int n) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kern, RowLdgShape::TT,
-                                                    RowLdgShape::smem) != cudaSuccess)
-    return 0;
-  if (per_sm < 1) per_sm = 1;
-  int x = (per_sm * current_device_sms() + n - 1) / n;
+  const int per_sm = resident_blocks<Kern>(RowLdgShape::TT, RowLdgShape::smem);
+  const int x = (per_sm * current_device_sms() + n - 1) / n;
   return x > RowLdgShape::N ? RowLdgShape::N : x;
 }
 
@@ -55,7 +51,6 @@ cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc,
     cudaError_t e = ensure_smem_attr<kern>(RowLdgShape::smem);
     if (e) return e;
     const int grid = row_ldg_grid<kern>(1);
-    if (grid < 1) return cudaErrorInvalidConfiguration;
     if (dep)
       return launch_dependent(kern, dim3(grid), dim3(RowLdgShape::TT), RowLdgShape::smem, st, jb, twc);
     kern<<<grid, RowLdgShape::TT, RowLdgShape::smem, st>>>(jb, twc);
@@ -68,10 +63,7 @@ cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc,
     if (e) return e;
     int grid = ((even_rows<T, SWEEP, BEAM>(N) ? M + 1 : N) + SH::G - 1) / SH::G;
     if constexpr (!SWEEP) {  // persistent blocks over the TMA row ring
-      int per_sm = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SH::threads, smem);
-      if (e) return e;
-      if (per_sm < 1) per_sm = 1;
+      const int per_sm = resident_blocks<kern>(SH::threads, smem);
       if (grid > per_sm * current_device_sms()) grid = per_sm * current_device_sms();
     }
     if (dep) return launch_dependent(kern, dim3(grid), dim3(SH::threads), smem, st, jb, twc, err);

@@ -246,10 +246,7 @@ cudaError_t launch_row_fx(const Jobs<RowJob<double>, K>& jb, int n, int scale, b
   constexpr size_t smem = S::smem(!SWEEP);
   cudaError_t e = ensure_smem_attr<kern>(smem);
   if (e) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, S::SH::threads, smem);
-  if (e) return e;
-  if (per_sm < 1) per_sm = 1;
+  const int per_sm = resident_blocks<kern>(S::SH::threads, smem);
   int x = (per_sm * current_device_sms() * (scale < 1 ? 1 : scale) + n - 1) / n;
   constexpr int rows = even_rows<double, SWEEP, BEAM>(S::N) ? S::M + 1 : S::N;
   if (x > (rows + S::G - 1) / S::G) x = (rows + S::G - 1) / S::G;
