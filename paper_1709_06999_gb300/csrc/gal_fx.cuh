@@ -159,39 +159,45 @@ __device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff80
 
 // ---------------------------------------------------------------------------
 // The transform: the Stockham plan of gal_fft3.cuh at radix 8, with its staged
-// factors in digits.  Those of the stages between the first and the last are
-// kept in shared memory (the first 8^(nstage-1) - 8 entries of the table).
+// factors in digits.  TAB: those of the stages before the last come from a copy in
+// shared memory (the first fx_ntab entries of the table); otherwise through L1.
+// The copy pays for rows of 1024 points and more, whose blocks have many (4096^2
+// image 277 against 281 us a call, 2048^2 98.6 against 100.6), and for columns of
+// 2048 and more, where it is made while the row pass ends (4096^2 277.6 against
+// 280.3); shorter ones do without (256 image 26.4 against 24.6, 1024 profile 82.4
+// against 81.7).
 // ---------------------------------------------------------------------------
-template <int L> struct FxPlan {
-  using P = P3<L, 8>;
-  static constexpr int ntab = P::nstage >= 3 ? ipowc(8, P::nstage - 1) - 8 : 0;
-};
-
-template <int L> __device__ __forceinline__ void fx_fill_tab(fxtw* tab, const fxtw* __restrict__ tws) {
-  for (int i = threadIdx.x; i < FxPlan<L>::ntab; i += blockDim.x) tab[i] = ldg_tw(tws + i);
+template <int L, int LMIN> constexpr int fx_ntab() {
+  return L >= LMIN ? ipowc(8, P3<L, 8>::nstage - 1) - 8 : 0;
 }
 
-template <int L, int ST> struct FxHead {
+template <int L, int ST, bool TAB> struct FxHead {
   using P = P3<L, 8>;
-  static __device__ __forceinline__ void run(fx2 (&v)[8], fx2* A, fx2* B, int t, const fxtw* tab) {
+  static __device__ __forceinline__ void run(fx2 (&v)[8], fx2* A, fx2* B, int t,
+                                             const fxtw* tws) {
     if constexpr (ST < P::nstage - 1) {
       constexpr int T = P::T, Ns = ipowc(8, ST);
       fx2* in = (ST % 2 == 1) ? A : B;
       fx2* out = (ST % 2 == 0) ? A : B;
       const int k = t & (Ns - 1);
       if constexpr (ST > 0) {
-        const fxtw* w = tab + (Ns - 8) + k;
+        const fxtw* w = tws + (Ns - 8) + k;
 #pragma unroll
         for (int r = 0; r < 8; ++r) v[r] = in[pad3<8>(t + r * T)];
+        if constexpr (TAB) {
 #pragma unroll
-        for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], w[(r - 1) * Ns]);
+          for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], w[(r - 1) * Ns]);
+        } else {
+#pragma unroll
+          for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], ldg_tw(w + (r - 1) * Ns));
+        }
       }
       bfly8(v);
       const int base = ST == 0 ? 9 * t : pad3<8>((t - k) * 8 + k);
 #pragma unroll
       for (int r = 0; r < 8; ++r) out[ST == 0 ? base + r : base + r * pad_step<8>(Ns)] = v[r];
       __syncthreads();
-      FxHead<L, ST + 1>::run(v, A, B, t, tab);
+      FxHead<L, ST + 1, TAB>::run(v, A, B, t, tws);
     }
   }
 };

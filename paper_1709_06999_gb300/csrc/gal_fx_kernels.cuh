@@ -23,9 +23,9 @@ template <int LG> struct FxRowShape {
   static constexpr int M = 1 << LG, N = 2 * M;
   using SH = Shape3<double, M, N, 128, 8>;
   static constexpr int G = SH::G, RS = SH::RS;
-  static constexpr int ntab = FxPlan<M>::ntab;
-  // header (barrier, reduction scratch, row scales), factor table, two work
-  // buffers, the image rows as they arrive
+  static constexpr int ntab = fx_ntab<M, 1024>();
+  // header (barrier, reduction scratch, row scales), factors, two work buffers, the
+  // image rows as they arrive
   static constexpr int kHead = 512;
   static constexpr size_t work = (size_t)G * RS * sizeof(fx2);
   static constexpr size_t smem(bool image) {
@@ -59,7 +59,7 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
   unsigned* red_sum = reinterpret_cast<unsigned*>(smem_raw + 96);
   int* row_q = reinterpret_cast<int*>(smem_raw + 192);              // per row of the group, <= 64
   fxtw* tab = reinterpret_cast<fxtw*>(smem_raw + S::kHead);
-  fx2* A0 = reinterpret_cast<fx2*>(smem_raw + S::kHead + (size_t)S::ntab * sizeof(fxtw));
+  fx2* A0 = reinterpret_cast<fx2*>(tab + S::ntab);
   fx2* B0 = A0 + G * RS;
   double* slot = reinterpret_cast<double*>(B0 + G * RS);
   static_assert(G <= 64 && SH::threads <= 512, "header");
@@ -85,7 +85,7 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
       issue(blockIdx.x);
     }
   }
-  fx_fill_tab<M>(tab, tws);
+  for (int i = threadIdx.x; i < S::ntab; i += blockDim.x) tab[i] = ldg_tw(tws + i);
   const Bounds bd = block_bounds(jb.rho2, jb.S, N);  // synchronises
   const bool pruned = P::nstage >= 2 && bd.Kc <= P::Nsl;
   if constexpr (BEAM) grid_dep_wait();  // the beam tables
@@ -124,7 +124,8 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
     if (t == 0) row_q[g] = sc.bad ? INT_MAX : sc.q;
     fx2* A = A0 + g * RS;
     fx2* B = B0 + g * RS;
-    FxHead<M, 0>::run(v, A, B, t, tab);
+    if constexpr (S::ntab > 0) FxHead<M, 0, true>::run(v, A, B, t, tab);
+    else FxHead<M, 0, false>::run(v, A, B, t, tws);
     fx2* in = last_input<M, 8>(A, B);
     if (!pruned) {
       fx_last_full<M>(v, in, t, tws);
@@ -159,7 +160,7 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
 template <int LG> struct FxColShape {
   static constexpr int N = 1 << LG;
   using SH = ColShape3<double, N, 8>;
-  static constexpr int ntab = FxPlan<N>::ntab;
+  static constexpr int ntab = fx_ntab<N, 2048>();
   static constexpr int kHead = 128 + 1024;  // reduction scratch, a scale per column
   static constexpr size_t smem =
       kHead + (size_t)ntab * sizeof(fxtw) + (size_t)2 * SH::G * SH::RS * sizeof(fx2);
@@ -183,10 +184,10 @@ col_fx_kernel(const __grid_constant__ Jobs<ColJob<double>, K> jobs, const double
   unsigned* red_sum = reinterpret_cast<unsigned*>(smem_raw + 64);
   int* col_q = reinterpret_cast<int*>(smem_raw + 128);
   fxtw* tab = reinterpret_cast<fxtw*>(smem_raw + S::kHead);
-  fx2* base = reinterpret_cast<fx2*>(smem_raw + S::kHead + (size_t)S::ntab * sizeof(fxtw));
+  fx2* base = reinterpret_cast<fx2*>(tab + S::ntab);
   static_assert(G <= 256 && SH::threads <= 512, "header");
   const int g = threadIdx.x / TT, t = threadIdx.x - g * TT;
-  fx_fill_tab<N>(tab, tws);
+  for (int i = threadIdx.x; i < S::ntab; i += blockDim.x) tab[i] = ldg_tw(tws + i);
   const Bounds bd = block_bounds(jb.rho2, jb.S, N);  // synchronises
   const int ncol = jb.full ? full_cols(bd, N).W : bd.Kc;
   const int kmax = N / 2 - bd.r0;
@@ -202,7 +203,8 @@ col_fx_kernel(const __grid_constant__ Jobs<ColJob<double>, K> jobs, const double
     for (int r = 0; r < 8; ++r) z[r] = act ? F1[f1_index(jb.even, N, c, t + r * TT)] : make_double2(0.0, 0.0);
     fx2 v[8];
     const FxScale sc = fx_load<TT>(z, v, red_max, red_sum);
-    FxHead<N, 0>::run(v, A, B, t, tab);
+    if constexpr (S::ntab > 0) FxHead<N, 0, true>::run(v, A, B, t, tab);
+    else FxHead<N, 0, false>::run(v, A, B, t, tws);
     fx2* in = last_input<N, 8>(A, B);
     auto value = [&](fx2 x, int q, bool bad) {
       return bad ? make_double2(fx_nan(), fx_nan()) : make_double2(fx_to(x.x, q), fx_to(x.y, q));
