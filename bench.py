@@ -104,7 +104,7 @@ def full_window_columns(Kc: int, N: int) -> int:
 
 # the sources that define the profiled kernels and their launch shapes
 KERNEL_SOURCES = ("gal_common.cuh", "gal_fft.cuh", "gal_fft2.cuh", "gal_fft3.cuh",
-                  "gal_fft3_launch.cuh", "gal_kernels.cuh", "gal_plane.cuh", "gal_tma.cuh",
+                  "gal_fft3_launch.cuh", "gal_fx.cuh", "gal_fx_kernels.cuh", "gal_kernels.cuh", "gal_plane.cuh", "gal_tma.cuh",
                   "gal_internal.h")
 
 

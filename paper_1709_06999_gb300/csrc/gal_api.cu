@@ -49,7 +49,10 @@ struct gal_ctx {
   unsigned* counter = nullptr;  // last-block-done counter (self-resetting)
   double* rho2 = nullptr;       // uv extent scratch for raw-pointer calls
   void* ext_state = nullptr;    // Launch::extent's: of those calls, and of registrations
-  double* reg_rho2 = nullptr;   // extent of the observation being registered (mapped host memory)
+  // registrations (a server's may come from several threads at once): the extent of
+  // the one that holds reg_mu, in mapped host memory
+  std::mutex reg_mu;
+  double* reg_rho2 = nullptr;
   double* uvrange = nullptr;    // min / max of u^2 + v^2 (image sizing)
   int* err = nullptr;           // index-check flag
   double* chi2_dev = nullptr;   // result slot for the host-buffer entry points
@@ -603,6 +606,7 @@ int data_create_t(gal_ctx* ctx, const T* u, const T* v, const T* re, const T* im
     // the extent comes back once, into mapped host memory: every call sizes its
     // window from it on the host and passes the kernels the result
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    std::lock_guard<std::mutex> lk(ctx->reg_mu);  // until the extent is read
     int s = stage(ctx, 0, st, [&] {
       return gal::Launch<T>::extent(u, v, M, ctx->reg_rho2,
                                     static_cast<char*>(ctx->ext_state) + gal::kExtentState,

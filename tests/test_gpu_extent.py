@@ -1,11 +1,13 @@
 """The uv extent pass: the farthest point decides which part of the spectrum is
 kept, so a point it missed would be sampled at the edge of a window too small."""
+import threading
+
 import numpy as np
 import pytest
 import torch
 
 import oracle
-from paper_1709_06999_gb300 import Context
+from paper_1709_06999_gb300 import Context, Request, Server
 
 pytestmark = pytest.mark.gpu
 # the visibility gates of the two paths (normwise)
@@ -62,3 +64,37 @@ def test_nonfinite_points_and_near_ties(dt):
         assert torch.isnan(got[17]).all()
         # a NaN point is left out of the extent, an infinite one keeps the whole plane
         assert torch.allclose(got[keep], ref[keep], rtol=0, atol=TOL[dt] * I.sum().item())
+
+
+def test_registrations_from_several_threads():
+    """Observations of different reach registered on one server at once: each
+    keeps its own extent (a chi-square equal to that of a context of its own)."""
+    n, dxy, M = 256, 1e-8, 40_001
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    I = torch.rand((n, n), generator=g, device="cuda")
+    data = []
+    for k in range(16):
+        a = torch.rand((5, M), generator=g, device="cuda")
+        r = (0.02 + 0.028 * k) / dxy
+        data.append([(a[0] - 0.5) * r, (a[1] - 0.5) * r, a[2], a[3], a[4]])
+    torch.cuda.synchronize()
+    server = Server(0)
+    for _ in range(4):
+        obs = [None] * len(data)
+        go = threading.Barrier(len(data))
+
+        def work(k):
+            go.wait()
+            obs[k] = server.add_data(*data[k])
+
+        ts = [threading.Thread(target=work, args=(k,)) for k in range(len(data))]
+        for t in ts:
+            t.start()
+        for t in ts:
+            t.join()
+        got = [server.wait(server.submit(Request(o, image=I, dxy=dxy)))[0] for o in obs]
+        ctx = Context(0)
+        want = [ctx.chi2_image(I, dxy, ctx.register(*d)).item() for d in data]
+        assert got == want
+    server.close()
