@@ -35,15 +35,21 @@ template <typename T, int LG, bool SWEEP> constexpr bool row_pairs_exist() {
 }
 constexpr int kRowPairsKc = 256;  // spans of the pruned last stage of 4096 points
 
-// A row pass that follows beam_table_kernel in the stream, or the extent pass
-// whose result it reads, is launched as its programmatic dependent (the kernels
-// wait for the tables, and block_bounds for the extent).
+// A row pass that follows beam_table_kernel in the stream (it waits for the tables
+// with its image copies in flight), or the extent pass whose result it reads, is
+// launched as its programmatic dependent.  So is a float image's row pass whose
+// grid takes every place on the GPU, whatever precedes it: it waits at its start,
+// before it reads or writes anything, so that only its launch overlaps, with the
+// previous call's gather if that is what precedes (4096 / 5e6 44.3 -> 41.5 us,
+// four copies of a 2048 / 2e6 model 38.8 -> 36.5 us, calls in a row).  A smaller
+// grid would crowd onto the SMs that come free first (1024 profiles, 129 and 257
+// blocks: 26.6 -> 28.5 and 82.0 -> 88.0 us), and the double pass lost 2 % too.
 template <typename T, int LG, bool SWEEP, bool BEAM, int V = FftV<T>::V, bool PAIRS = false>
 cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc, int* err,
                              cudaStream_t st) {
   using C = cplx_t<T>;
   constexpr int M = 1 << LG, N = 2 * M;
-  const bool dep = BEAM || jb.j[0].rho2.rho2;
+  bool dep = BEAM || jb.j[0].rho2.rho2;
   if constexpr (sizeof(T) == 8) {  // double rows: on integers
     return launch_row_fx<LG, SWEEP, 1, BEAM>(jb, 1, 1, dep, twc, err, st);
   } else if constexpr (row_ldg_shape<T, LG, SWEEP, V>()) {  // float rows of 4096 pixels
@@ -51,10 +57,7 @@ cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc,
     cudaError_t e = ensure_smem_attr<kern>(RowLdgShape::smem);
     if (e) return e;
     const int grid = row_ldg_grid<kern>(1);
-    if (dep)
-      return launch_dependent(kern, dim3(grid), dim3(RowLdgShape::TT), RowLdgShape::smem, st, jb, twc);
-    kern<<<grid, RowLdgShape::TT, RowLdgShape::smem, st>>>(jb, twc);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3(grid), dim3(RowLdgShape::TT), RowLdgShape::smem, st, jb, twc);
   } else {
     using SH = Shape3<T, M, N, row_min_threads(PAIRS), V>;
     constexpr auto kern = row_fft3_kernel<T, LG, !SWEEP, SWEEP, 1, BEAM, row_min_threads(PAIRS), 2, V>;
@@ -64,7 +67,9 @@ cudaError_t launch_row3_kern(const Jobs<RowJob<T>, 1>& jb, const cplx_t<T>* twc,
     int grid = ((even_rows<T, SWEEP, BEAM>(N) ? M + 1 : N) + SH::G - 1) / SH::G;
     if constexpr (!SWEEP) {  // persistent blocks over the TMA row ring
       const int per_sm = resident_blocks<kern>(SH::threads, smem);
-      if (grid > per_sm * current_device_sms()) grid = per_sm * current_device_sms();
+      const int places = per_sm * current_device_sms();
+      dep = dep || grid >= places;
+      if (grid > places) grid = places;
     }
     if (dep) return launch_dependent(kern, dim3(grid), dim3(SH::threads), smem, st, jb, twc, err);
     kern<<<grid, SH::threads, smem, st>>>(jb, twc, err);

@@ -544,7 +544,11 @@ __global__ void __launch_bounds__(Shape3<T, (1 << LG), (2 << LG), MINT, VR>::thr
 row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>* __restrict__ tw,
                 int* __restrict__ err) {
   using C = cplx_t<T>;
-  grid_dep_launch();  // the column pass may be scheduled as our blocks retire
+  // first all that came before in the stream (the kernels scheduled next read the
+  // points before they wait for us); then the column pass may be scheduled as our
+  // blocks retire
+  if constexpr (!BEAM) grid_dep_wait();
+  grid_dep_launch();
   const RowJob<T>& jb = jobs.j[K == 1 ? 0 : blockIdx.y];
   const T* __restrict__ image = jb.image;
   const T* __restrict__ I = jb.I;
@@ -742,7 +746,11 @@ row_fft3_ldg_kernel(const __grid_constant__ Jobs<RowJob<float>, K> jobs, const f
   using P = SH::P;
   constexpr int M = SH::M, N = SH::N, V = SH::V, TT = SH::TT, RS = SH::RS;
   static_assert(P::nstage == 3 && P::rlast == 8 && P::Nsl == 256 && TT == 128, "shape");
-  grid_dep_launch();  // the column pass may be scheduled as our blocks retire
+  // first all that came before in the stream (the kernels scheduled next read the
+  // points before they wait for us); then the column pass may be scheduled as our
+  // blocks retire
+  if constexpr (!BEAM) grid_dep_wait();
+  grid_dep_launch();
   const RowJob<float>& jb = jobs.j[K == 1 ? 0 : blockIdx.y];
   const float* __restrict__ image = jb.image;
   const float* __restrict__ beam = BEAM ? jb.beam : nullptr;
@@ -1856,6 +1864,9 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
     tab = sct;
   }
   grid_dep_wait();  // the window is the column pass's output
+  // From here on the column pass is over, so the next call's row pass, which writes
+  // F1, may be scheduled as our blocks retire.
+  if constexpr (K == 1) grid_dep_launch();
   C* sw = nullptr;
   bool win_ok = true;
   if constexpr (SMEM) {
