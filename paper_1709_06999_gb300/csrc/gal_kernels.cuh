@@ -670,7 +670,10 @@ row_fft3_kernel(const __grid_constant__ Jobs<RowJob<T>, K> jobs, const cplx_t<T>
       // stage 0 writes the work buffer; the slot is reused from stage 1 on,
       // after the barrier that ends stage 0
       transform(v, work + (size_t)g * RS, slot, grp * G + g);
-      __syncthreads();  // every read of this slot is done
+      // the refill goes through the async proxy, which a barrier alone does not
+      // order after the transform's loads and stores in the slot: every thread fences
+      fence_proxy_async_smem();
+      __syncthreads();  // every use of this slot is done
       if (threadIdx.x == 0) issue(it + NSLOT);
     }
   } else {
