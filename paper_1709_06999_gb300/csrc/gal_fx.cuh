@@ -4,15 +4,28 @@
 // multiply-adds per second), but 64 integer additions and 32 multiply-adds of
 // 32 x 32 -> 64 bits (7.6e12 per second measured).  A double transform is
 // therefore done on integers: the values of one sequence share one power of
-// two (a block exponent), chosen from the sum of their magnitudes so that no
-// partial sum of the transform can overflow, and keep 60 bits below that sum.
-// A double keeps 53 bits below each value, so this is no less precise: every
-// rounding of the transform is at 2^-60 of a bound on its outputs.  Inputs and
+// two (a block exponent) that grows with the transform.  After s stages of radix
+// 8 a value is at most min(8^s largest modulus, sum of magnitudes), both known
+// at the load; the values enter each stage below 2^60 of that bound, grow by up
+// to 8 in its butterflies, and are shifted back, by as many bits as the bound
+// grew, inside the next product.  Each stage thus rounds at 2^-60 of what the
+// values can be at that stage: the largest inputs keep all 53 bits, and the
+// roundings of the early stages are far below those of the last.  Inputs and
 // outputs in memory stay doubles.
+//
+// Error against 64 bits, root mean square over the rms spectrum, after row and
+// column pass within 24 cells of the origin (the same steps on a CPU against an
+// extended-precision transform; the FP64 plan in brackets): noise 1.0e-16
+// (2.9e-16) at 512^2, 1.2e-16 (3.3e-16) at 2048^2, 1.4e-16 (3.5e-16) at 4096^2;
+// a smooth source 6.0e-17 (1.3e-16), 6.0e-17 (1.3e-16), 6.1e-17 (1.5e-16);
+// positive random pixels 8.0e-17 (8.9e-17), 8.9e-17 (9.0e-17), 4.3e-17
+// (4.4e-17).  One scale for all stages, taken from the sum, had 8.4e-16, 7.6e-15
+// and 2.9e-14 for the noise, growing with the side.
 //
 // A complex product by a unit-modulus factor takes 12 multiply-adds (three
 // 32 x 32 products per real product: high x high and the two cross terms, the
-// low x low term being below the last bit).
+// low x low term being a quarter of the last bit at most where the values use
+// all 63 bits, as in the stages).
 #pragma once
 
 #include "gal_common.cuh"
@@ -42,6 +55,22 @@ __device__ __forceinline__ fxtw fx_factor(double x, double y) {  // |x|, |y| <= 
   fx_digits(__double2ll_rn(y * k62), w.yh, w.yl);
   return w;
 }
+// The staged factors of the transforms: the same in units of 2^-61, and 1 is one
+// unit short.  A product by 1 is a shift, whose ties are frequent; rounded up
+// like all others they would bias every value the same way, which adds up in the
+// sums (24 times the other errors at the origin of a 4096^2 spectrum).  One unit
+// less makes them round towards zero.
+__device__ __forceinline__ fxtw fx_stage_factor(double x, double y) {
+  constexpr long long one = 1ll << 61;
+  auto units = [](double a) {
+    const long long q = __double2ll_rn(a * (double)one);
+    return q == one ? q - 1 : q == -one ? q + 1 : q;
+  };
+  fxtw w;
+  fx_digits(units(x), w.xh, w.xl);
+  fx_digits(units(y), w.yh, w.yl);
+  return w;
+}
 
 __device__ __forceinline__ long long madw(int a, int b, long long c) {
   return (long long)a * (long long)b + c;
@@ -53,7 +82,7 @@ __device__ __forceinline__ void fx_split(long long a, int& h, int& l) {
 }
 constexpr long long kFxHalf = 0x80000000ll;  // rounds the cross terms to nearest
 
-// hi 64 bits of a w (a |a| < 2^61, w in units of 2^-62): a w / 4
+// hi 64 bits of a w (|a| < 2^62.5): a w / 4 for w in units of 2^-62
 __device__ __forceinline__ long long fx_mul_q(long long a, int wh, int wl) {
   int h, l;
   fx_split(a, h, l);
@@ -64,7 +93,8 @@ __device__ __forceinline__ long long fx_mul(long long a, int wh, int wl) {
   return fx_mul_q(a, wh, wl) << 2;
 }
 
-// a w / 4 for complex a (components below 2^62, modulus below 2^61.5)
+// a w / 4 for complex a (modulus below 2^62); for a staged factor (fx_stage_factor)
+// a w / 8 (modulus below 2^63): the cross terms' sum stays below 2^63 either way
 __device__ __forceinline__ fx2 fx_cmul_q(fx2 a, const fxtw& w) {
   int xh, xl, yh, yl;
   fx_split(a.x, xh, xl);
@@ -82,10 +112,20 @@ __device__ __forceinline__ fxtw ldg_tw(const fxtw* p) {
   const int4 v = __ldg(reinterpret_cast<const int4*>(p));
   return fxtw{v.x, v.y, v.z, v.w};
 }
-// x / sqrt 2 (bfly8): 2^61.5 to the nearest, in digits
+// x / sqrt 2 (bfly8), |x| < 2^62: 2^62.5 to the nearest, in digits
 template <> __device__ __forceinline__ long long mul_sqrt_half<long long>(long long x) {
-  return fx_mul(x, 0x2D413CCD, -25716447);
+  return fx_mul_q(x << 1, 0x5A82799A, -51432894);
 }
+// a w 2^(p - 3) for a staged factor w; the modulus of a is below 2^(63 - p)
+__device__ __forceinline__ fx2 fx_stage_mul(fx2 a, const fxtw& w, int p) {
+  return fx_cmul_q(fx2{(long long)((unsigned long long)a.x << p), (long long)((unsigned long long)a.y << p)}, w);
+}
+// a / 2^g to the nearest, ties towards zero (see fx_stage_factor), 0 <= g <= 3
+__device__ __forceinline__ long long fx_shr(long long a, int g) {
+  const unsigned up = (unsigned)((unsigned long long)a >> 63) & (g > 0 ? 1u : 0u);
+  return (long long)((unsigned long long)a + (unsigned)((((1 << g) - 1) >> 1) + up)) >> g;
+}
+__device__ __forceinline__ fx2 fx_shr(fx2 a, int g) { return fx2{fx_shr(a.x, g), fx_shr(a.y, g)}; }
 
 // ---------------------------------------------------------------------------
 // doubles to a common power of two and back
@@ -121,41 +161,65 @@ __device__ __forceinline__ long long fx_sign(long long v, double x) {
 __device__ __forceinline__ unsigned fx_ebits(double x) {
   return (unsigned)__double2hiint(x) & 0x7fffffffu;
 }
-// |x| rounded up, in units of 2^(E - 1040), E >= its exponent: at most 2^18 + 1
-__device__ __forceinline__ unsigned fx_ceil_units(double x, int E) {
-  const unsigned hi = (unsigned)__double2hiint(x);
+// the double of high word hi rounded up, in units of 2^(E - 1040), E >= its
+// exponent: at most 2^18 + 1
+__device__ __forceinline__ unsigned fx_ceil_units(unsigned hi, int E) {
   const int be = (int)((hi >> 20) & 0x7ffu);
   const unsigned mh = (hi & 0xfffffu) + ((unsigned)min(be, 1) << 20);
   return shr_clamp(mh, E - max(be, 1) + 3) + 1u;
 }
 
-// Block exponent of a sequence: E is its largest biased exponent (>= 1), T the
-// sum of fx_ceil_units over its real values.  The sum of magnitudes is then
-// below 2^(bits + E - 1040); fixed-point value f stands for f 2^q, with every
-// partial sum of the transform below 2^60.
+// Block exponent of a sequence: E is its largest biased exponent (>= 1), C the
+// largest and T the sum of fx_ceil_units over its real values.  The moduli are
+// below 2^mb and their sum below 2^bits in the same units; fixed-point value f
+// stands for f 2^q.
 struct FxScale {
   int D;     // right shift of a 63-bit significand of exponent e: D - e
-  int q;     // exponent of one unit
+  int q;     // exponent of one unit: moduli start below 2^60 units
+  int left;  // bits by which the transform's values can grow beyond that
   bool bad;  // the sequence holds an infinity or a NaN
+  // The shift before a stage whose inputs were just stored: as much as the values
+  // may have grown in the stage before (3 bits: radix 8).
+  __device__ __forceinline__ int stage() {
+    const int g = min(3, left);
+    left -= g;
+    q += g;
+    return g;
+  }
 };
-__device__ __forceinline__ FxScale fx_scale(int E, unsigned T) {
+__device__ __forceinline__ FxScale fx_scale(int E, unsigned C, unsigned T) {
   const int bits = max(32 - __clz((int)T), 16);
-  return FxScale{bits + E - 15, bits + E - 1100, E >= 0x7ff};
+  const int mb = max(32 - __clz((int)(C + (C >> 1))), 16);  // 3/2 > sqrt 2: modulus from components
+  const int s0 = min(mb, bits);
+  return FxScale{s0 + E - 15, s0 + E - 1100, bits - s0, E >= 0x7ff};
 }
 __device__ __forceinline__ long long fx_from(double x, const FxScale& s) {
   int e;
   const unsigned long long m = fx_mant(x, e);
   return fx_sign((long long)((shr64_clamp(m << 10, s.D - e - 1) + 1ull) >> 1), x);
 }
-// v 2^q, rounded once (twice only where the result is subnormal)
-__device__ __forceinline__ double fx_to(long long v, int q) {
-  const double y = __ll2double_rn(v);
-  if (q >= -1021 && q <= 959)  // 1 <= |y| < 2^63 or y = 0: the exponent cannot leave its field
-    return v ? __hiloint2double(__double2hiint(y) + (q << 20), __double2loint(y)) : 0.0;
-  const int a = q / 2, b = q - a;
-  return y * __hiloint2double((1023 + a) << 20, 0) * __hiloint2double((1023 + b) << 20, 0);
-}
 __device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
+
+// v 2^q as doubles, |v.x|, |v.y| < 2^63, each rounded once (twice only where the
+// result is subnormal); NaN for q = kFxBad.  One branch for exponents that could
+// leave their field (two, one to a component: 4096^2 image 284.3 against 282.2 us,
+// 1024 profile 82.4 against 81.1).
+constexpr int kFxBad = 4096;
+__device__ __forceinline__ double2 fx_to(fx2 v, int q) {
+  const double x = __ll2double_rn(v.x), y = __ll2double_rn(v.y);
+  if ((unsigned)(q + 1021) > 1980u) {
+    if (q == kFxBad) return make_double2(fx_nan(), fx_nan());
+    const int a = q / 2, b = q - a;
+    const double f = __hiloint2double((1023 + a) << 20, 0), g = __hiloint2double((1023 + b) << 20, 0);
+    return make_double2(x * f * g, y * f * g);
+  }
+  // 1 <= |x| <= 2^63 or x = 0
+  auto scaled = [&](double d) {
+    const int h = __double2hiint(d);
+    return __hiloint2double(h + (h ? q << 20 : 0), __double2loint(d));
+  };
+  return make_double2(scaled(x), scaled(y));
+}
 
 // ---------------------------------------------------------------------------
 // The transform: the Stockham plan of gal_fft3.cuh at radix 8, with its staged
@@ -174,7 +238,7 @@ template <int L, int LMIN> constexpr int fx_ntab() {
 template <int L, int ST, bool TAB> struct FxHead {
   using P = P3<L, 8>;
   static __device__ __forceinline__ void run(fx2 (&v)[8], fx2* A, fx2* B, int t,
-                                             const fxtw* tws) {
+                                             const fxtw* tws, FxScale& sc) {
     if constexpr (ST < P::nstage - 1) {
       constexpr int T = P::T, Ns = ipowc(8, ST);
       fx2* in = (ST % 2 == 1) ? A : B;
@@ -184,12 +248,14 @@ template <int L, int ST, bool TAB> struct FxHead {
         const fxtw* w = tws + (Ns - 8) + k;
 #pragma unroll
         for (int r = 0; r < 8; ++r) v[r] = in[pad3<8>(t + r * T)];
+        const int g = sc.stage(), p = 3 - g;
+        v[0] = fx_shr(v[0], g);
         if constexpr (TAB) {
 #pragma unroll
-          for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], w[(r - 1) * Ns]);
+          for (int r = 1; r < 8; ++r) v[r] = fx_stage_mul(v[r], w[(r - 1) * Ns], p);
         } else {
 #pragma unroll
-          for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], ldg_tw(w + (r - 1) * Ns));
+          for (int r = 1; r < 8; ++r) v[r] = fx_stage_mul(v[r], ldg_tw(w + (r - 1) * Ns), p);
         }
       }
       bfly8(v);
@@ -197,15 +263,25 @@ template <int L, int ST, bool TAB> struct FxHead {
 #pragma unroll
       for (int r = 0; r < 8; ++r) out[ST == 0 ? base + r : base + r * pad_step<8>(Ns)] = v[r];
       __syncthreads();
-      FxHead<L, ST + 1, TAB>::run(v, A, B, t, tws);
+      FxHead<L, ST + 1, TAB>::run(v, A, B, t, tws, sc);
     }
   }
 };
 
+// The last stage's shift g of its inputs (FxScale::stage; none if it is the only
+// stage) and the bits r its outputs may exceed 2^60 by.
+struct FxLast {
+  int g, r;
+};
+template <int L> __device__ __forceinline__ FxLast fx_last(FxScale& sc) {
+  using P = P3<L, 8>;
+  const int g = P::nstage > 1 ? sc.stage() : 0;
+  return FxLast{g, min(ilog2c(P::rlast), sc.left)};
+}
 // last stage, complete: v[q R + r] <- X[t + q T + r L / R]
 template <int L>
 __device__ __forceinline__ void fx_last_full(fx2 (&v)[8], const fx2* in, int t,
-                                             const fxtw* __restrict__ tws) {
+                                             const fxtw* __restrict__ tws, int g) {
   using P = P3<L, 8>;
   constexpr int R = P::rlast, T = P::T;
   if constexpr (P::nstage == 1) {
@@ -216,9 +292,10 @@ __device__ __forceinline__ void fx_last_full(fx2 (&v)[8], const fx2* in, int t,
       const int b = t + q * T;
 #pragma unroll
       for (int r = 0; r < R; ++r) v[q * R + r] = in[pad3<8>(b + r * (L / R))];
+      v[q * R] = fx_shr(v[q * R], g);
 #pragma unroll
-      for (int r = 1; r < R; ++r) 
-        v[q * R + r] = cmul(v[q * R + r], ldg_tw(tws + (P::Nsl - 8) + (r - 1) * P::Nsl + b));
+      for (int r = 1; r < R; ++r)
+        v[q * R + r] = fx_stage_mul(v[q * R + r], ldg_tw(tws + (P::Nsl - 8) + (r - 1) * P::Nsl + b), 3 - g);
       bflyR<R>(&v[q * R]);
     }
   }
@@ -227,27 +304,30 @@ __device__ __forceinline__ void fx_last_full(fx2 (&v)[8], const fx2* in, int t,
 // X[j] and X[L - j] only (pruned_pair3)
 template <int L>
 __device__ __forceinline__ void fx_pruned_pair(const fx2* in, int j, const fxtw* __restrict__ tws,
-                                               fx2& xj, fx2& xmj) {
+                                               int g, fx2& xj, fx2& xmj) {
   using P = P3<L, 8>;
   constexpr int R = P::rlast, Ns = P::Nsl;
   const int jb = j == 0 ? Ns : j;
   const int ba = pad3<8>(j), bb = -jb + ((-jb) >> P::lv);
-  fx2 a = in[ba], b = in[bb + pad_step<8>(Ns)];
+  fx2 a = fx_shr(in[ba], g), b = fx_shr(in[bb + pad_step<8>(Ns)], g);
 #pragma unroll
   for (int r = 1; r < R; ++r) {
     const fxtw w = ldg_tw(tws + (Ns - 8) + (r - 1) * Ns + j);
-    a = cadd(a, cmul(in[ba + r * pad_step<8>(Ns)], w));
-    b = cadd(b, cmul(in[bb + (r + 1) * pad_step<8>(Ns)], cconj(w)));
+    a = cadd(a, fx_stage_mul(in[ba + r * pad_step<8>(Ns)], w, 3 - g));
+    b = cadd(b, fx_stage_mul(in[bb + (r + 1) * pad_step<8>(Ns)], cconj(w), 3 - g));
   }
   xj = a;
   xmj = j == 0 ? a : b;
 }
 
 // 2 X_k of a real row from the bins Z_k, Z_{M-k} of its packed transform
-// (r2c_unpack without the halving, which goes into the exponent)
+// (r2c_unpack without the halving, which goes into the exponent); the bins below
+// 2^60, w in units of 2^-62
 __device__ __forceinline__ fx2 fx_r2c_unpack2(fx2 zk, fx2 zmk, const fxtw& w) {
   const fx2 b = cconj(zmk);
-  return cadd(cadd(zk, b), cmul(cmul_mi(csub(zk, b)), w));
+  const fx2 d = cmul_mi(csub(zk, b));
+  const fx2 p = fx_cmul_q(fx2{d.x << 1, d.y << 1}, w);
+  return cadd(cadd(zk, b), fx2{p.x << 1, p.y << 1});
 }
 
 // Largest and sum over the TT threads of one sequence (threads t0 .. t0+TT-1
@@ -279,11 +359,13 @@ __device__ __forceinline__ FxScale fx_load(const double2 (&z)[8], fx2 (&v)[8], u
   unsigned h = 0;
 #pragma unroll
   for (int r = 0; r < 8; ++r) h = max(h, max(fx_ebits(z[r].x), fx_ebits(z[r].y)));
-  const int E = max((int)(fx_group<TT, true>(h, red_max) >> 20), 1);
+  h = fx_group<TT, true>(h, red_max);
+  const int E = max((int)(h >> 20), 1);
+  auto units = [&](double x) { return fx_ceil_units((unsigned)__double2hiint(x), E); };
   unsigned s = 0;
 #pragma unroll
-  for (int r = 0; r < 8; ++r) s += fx_ceil_units(z[r].x, E) + fx_ceil_units(z[r].y, E);
-  const FxScale sc = fx_scale(E, fx_group<TT, false>(s, red_sum));
+  for (int r = 0; r < 8; ++r) s += units(z[r].x) + units(z[r].y);
+  const FxScale sc = fx_scale(E, fx_ceil_units(h, E), fx_group<TT, false>(s, red_sum));
 #pragma unroll
   for (int r = 0; r < 8; ++r) v[r] = fx2{fx_from(z[r].x, sc), fx_from(z[r].y, sc)};
   return sc;
@@ -297,7 +379,9 @@ __device__ __forceinline__ FxScale fx_load(const double2 (&z)[8], fx2 (&v)[8], u
 constexpr int kSinCos = 1024;  // table of W_1024^k = cos - i sin at k / 1024 turns
 constexpr int kPosBits = 50;   // fraction bits of a grid position
 
-// grid offset x in units of 2^-50, to nearest; |x| >= 4096 (beyond every grid) saturates
+// grid offset x in units of 2^-50, to nearest; |x| >= 4096 (beyond every grid)
+// saturates.  Coarser than the double itself within 4 cells of the origin, by
+// 2^-51 of the step between two nodes at most.
 __device__ __forceinline__ long long fx_pos(double x) {
   int e;
   const unsigned long long m = fx_mant(x, e);
@@ -342,7 +426,8 @@ __device__ __forceinline__ fx2 fx_cos_sin(unsigned long long p, const fxtw* tab)
 }
 
 // Nodes of one cell at the power of two of the largest of their 8 values, E its
-// biased exponent: 2^59 <= |largest| < 2^60, one unit 2^(E - 1082).
+// biased exponent: 2^59 <= |largest| < 2^60, one unit 2^(E - 1082); a smaller node
+// is cut at that unit, 2^-59 of the largest.
 __device__ __forceinline__ long long fx_node(double x, int E) {
   int e;
   const unsigned long long m = fx_mant(x, e);

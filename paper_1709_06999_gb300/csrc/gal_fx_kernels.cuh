@@ -7,8 +7,6 @@
 // 41 -> 12 us, of 2048 x 413 66 -> 19 us.
 #pragma once
 
-#include <climits>
-
 #include "gal_fx.cuh"
 #include "gal_kernels.cuh"
 
@@ -57,7 +55,7 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   unsigned* red_max = reinterpret_cast<unsigned*>(smem_raw + 32);   // one per warp, <= 16
   unsigned* red_sum = reinterpret_cast<unsigned*>(smem_raw + 96);
-  int* row_q = reinterpret_cast<int*>(smem_raw + 192);              // per row of the group, <= 64
+  int* row_q = reinterpret_cast<int*>(smem_raw + 192);              // scale per row of the group, <= 64
   fxtw* tab = reinterpret_cast<fxtw*>(smem_raw + S::kHead);
   fx2* A0 = reinterpret_cast<fx2*>(tab + S::ntab);
   fx2* B0 = A0 + G * RS;
@@ -120,15 +118,21 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
       for (int r = 0; r < 8; ++r) z[r] = beam_pair(z[r], beam, N, row, t + r * TT);
     }
     fx2 v[8];
-    const FxScale sc = fx_load<TT>(z, v, red_max, red_sum);
-    if (t == 0) row_q[g] = sc.bad ? INT_MAX : sc.q;
+    FxScale sc = fx_load<TT>(z, v, red_max, red_sum);
     fx2* A = A0 + g * RS;
     fx2* B = B0 + g * RS;
-    if constexpr (S::ntab > 0) FxHead<M, 0, true>::run(v, A, B, t, tab);
-    else FxHead<M, 0, false>::run(v, A, B, t, tws);
+    if (t == 0) {  // of the last stage: shift, growth, exponent of its outputs
+      FxScale end = sc;
+#pragma unroll
+      for (int i = 1; i < P::nstage - 1; ++i) end.stage();
+      const FxLast l = fx_last<M>(end);
+      row_q[g] = sc.bad ? (kFxBad + 1) * 16 : end.q * 16 + l.g * 4 + l.r;
+    }
+    if constexpr (S::ntab > 0) FxHead<M, 0, true>::run(v, A, B, t, tab, sc);
+    else FxHead<M, 0, false>::run(v, A, B, t, tws, sc);
     fx2* in = last_input<M, 8>(A, B);
     if (!pruned) {
-      fx_last_full<M>(v, in, t, tws);
+      fx_last_full<M>(v, in, t, tws, fx_last<M>(sc).g);
       in = in == A ? B : A;
       store_full<M, 8>(v, in, t);
       __syncthreads();
@@ -141,17 +145,16 @@ row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double
       const int k = o / G, gg = o - k * G;
       if (EVEN && grp * G + gg > M) continue;
       const fx2* x = in0 + gg * RS;
+      const int rq = row_q[gg], r = rq & 3, q = (rq >> 4) + r;
       fx2 zk, zmk;
       if (pruned) {
-        fx_pruned_pair<M>(x, k, tws, zk, zmk);
+        fx_pruned_pair<M>(x, k, tws, (rq >> 2) & 3, zk, zmk);
       } else {
         zk = x[pad3<8>(k & (M - 1))];
         zmk = x[pad3<8>((M - k) & (M - 1))];
       }
-      const fx2 X2 = fx_r2c_unpack2(zk, zmk, ldg_tw(tw + k));
-      const int q = row_q[gg];
-      F1[(size_t)k * LD + grp * G + gg] =
-          q == INT_MAX ? make_double2(fx_nan(), fx_nan()) : make_double2(fx_to(X2.x, q - 1), fx_to(X2.y, q - 1));
+      const fx2 X2 = fx_r2c_unpack2(fx_shr(zk, r), fx_shr(zmk, r), ldg_tw(tw + k));
+      F1[(size_t)k * LD + grp * G + gg] = fx_to(X2, q - 1);
     }
     __syncthreads();  // every read of the work buffers and scales is done
   }
@@ -202,35 +205,32 @@ col_fx_kernel(const __grid_constant__ Jobs<ColJob<double>, K> jobs, const double
 #pragma unroll
     for (int r = 0; r < 8; ++r) z[r] = act ? F1[f1_index(jb.even, N, c, t + r * TT)] : make_double2(0.0, 0.0);
     fx2 v[8];
-    const FxScale sc = fx_load<TT>(z, v, red_max, red_sum);
-    if constexpr (S::ntab > 0) FxHead<N, 0, true>::run(v, A, B, t, tab);
-    else FxHead<N, 0, false>::run(v, A, B, t, tws);
+    FxScale sc = fx_load<TT>(z, v, red_max, red_sum);
+    if constexpr (S::ntab > 0) FxHead<N, 0, true>::run(v, A, B, t, tab, sc);
+    else FxHead<N, 0, false>::run(v, A, B, t, tws, sc);
+    const int lg = fx_last<N>(sc).g, cq = sc.bad ? kFxBad : sc.q;
     fx2* in = last_input<N, 8>(A, B);
-    auto value = [&](fx2 x, int q, bool bad) {
-      return bad ? make_double2(fx_nan(), fx_nan()) : make_double2(fx_to(x.x, q), fx_to(x.y, q));
-    };
     if (pruned) {
       for (int j = t; j <= kmax; j += TT) {
         fx2 xj, xmj;
-        fx_pruned_pair<N>(in, j, tws, xj, xmj);
+        fx_pruned_pair<N>(in, j, tws, lg, xj, xmj);
         if (act) {
-          Gw[(size_t)(kmax + j) * ncol + c] = value(xj, sc.q, sc.bad);
-          if (j > 0) Gw[(size_t)(kmax - j) * ncol + c] = value(xmj, sc.q, sc.bad);
+          Gw[(size_t)(kmax + j) * ncol + c] = fx_to(xj, cq);
+          if (j > 0) Gw[(size_t)(kmax - j) * ncol + c] = fx_to(xmj, cq);
         }
       }
     } else {
-      fx_last_full<N>(v, in, t, tws);
+      fx_last_full<N>(v, in, t, tws, lg);
       fx2* o = in == A ? B : A;
       store_full<N, 8>(v, o, t);
-      if (t == 0) col_q[g] = sc.bad ? INT_MAX : sc.q;
+      if (t == 0) col_q[g] = cq;
       __syncthreads();
       const fx2* o0 = o - (size_t)g * RS;
       for (int q = threadIdx.x; q < bd.nrw * G; q += G * TT) {
         const int rr = q / G, gg = q - rr * G;
         if (c0 + gg < ncol)
           Gw[(size_t)rr * ncol + c0 + gg] =
-              value(o0[(size_t)gg * RS + pad3<8>((bd.r0 + rr + N / 2) & (N - 1))], col_q[gg],
-                    col_q[gg] == INT_MAX);
+              fx_to(o0[(size_t)gg * RS + pad3<8>((bd.r0 + rr + N / 2) & (N - 1))], col_q[gg]);
       }
     }
     __syncthreads();

@@ -54,15 +54,15 @@ __global__ void twiddle_kernel(cplx_t<T>* __restrict__ tw, int N) {
     put(tw + TwTab<T, 8>::row(N), N / 2 - 8, row(8));
   } else {
     put(tw + TwTab<T, 8>::col(N), N - 8, col(8));
-    auto put_fx = [&](size_t off, int n, auto&& exponent) {
+    auto put_fx = [&](size_t off, int n, auto&& exponent, bool staged) {
       for (int k = t0; k < n; k += stride) {
         const double2 w = factor(exponent(k));
-        reinterpret_cast<fxtw*>(tw + off)[k] = fx_factor(w.x, w.y);
+        reinterpret_cast<fxtw*>(tw + off)[k] = staged ? fx_stage_factor(w.x, w.y) : fx_factor(w.x, w.y);
       }
     };
-    put_fx(TwTab<T, 8>::fx(N), N, plain);
-    put_fx(TwTab<T, 8>::fx_col(N), N - 8, col(8));
-    put_fx(TwTab<T, 8>::fx_row(N), N / 2 - 8, row(8));
+    put_fx(TwTab<T, 8>::fx(N), N, plain, false);
+    put_fx(TwTab<T, 8>::fx_col(N), N - 8, col(8), true);
+    put_fx(TwTab<T, 8>::fx_row(N), N / 2 - 8, row(8), true);
   }
 }
 
@@ -1547,30 +1547,26 @@ __device__ __forceinline__ double2 sample_point(const cplx_t<double>* __restrict
   auto node = [&](double2 a) { return fx2{fx_node(a.x, E), fx_node(a.y, E)}; };
   fx2 V = fx_lerp(fx_lerp(node(g00), node(g01), cfh, cfl), fx_lerp(node(g10), node(g11), cfh, cfl), rfh, rfl);
   if (neg) V.y = -V.y;
-  const int q = E - 1082;
   // V turned by one offset's phase
   auto turned = [&](double phx, double phy) {
     const double ph = u * phx + v * phy;
-    bad = bad || fx_nonfinite(ph);
     const fx2 e = fx_cos_sin(fx_turns(ph), tab);
     fxtw f;
     fx_digits(e.x, f.xh, f.xl);
     fx_digits(e.y, f.yh, f.yl);
-    const fx2 R = cmul(V, f);
-    return make_double2(fx_to(R.x, q), fx_to(R.y, q));
+    return fx_to(cmul(V, f), bad || fx_nonfinite(ph) ? kFxBad : E - 1082);
   };
-  double2 out;
   if constexpr (MULTI) {  // (one copy of amplitude 1 is the single call, bit for bit)
-    out = make_double2(0.0, 0.0);
+    double2 out = make_double2(0.0, 0.0);
     for (int k = 0; k < mp->K; ++k) {
       const double2 R = turned(mp->phx[k], mp->phy[k]);
       out.x = fma(mp->amp[k], R.x, out.x);
       out.y = fma(mp->amp[k], R.y, out.y);
     }
+    return out;
   } else {
-    out = turned(p.phx, p.phy);
+    return turned(p.phx, p.phy);
   }
-  return bad ? make_double2(fx_nan(), fx_nan()) : out;
 }
 
 // Sum of one double per lane, fixed order, valid in lane 0.  (A warp of zeros has
