@@ -1580,7 +1580,7 @@ __device__ __forceinline__ double warp_sum(double x) {
 }
 
 // per-thread compensated accumulators.  A block's total is formed in two steps:
-// put() leaves each warp's total in a slot of 32 doubles, and after a barrier one
+// put() leaves each warp's total in its place in a slot of 32 doubles, and after a barrier one
 // warp's cross() adds a slot's entries (valid in lane 0).
 struct AccF {  // Kahan: s holds the sum, c the negated lost low-order part
   float s = 0.f, c = 0.f;
@@ -1605,13 +1605,13 @@ struct AccF {  // Kahan: s holds the sum, c the negated lost low-order part
     }
     return a;
   }
-  __device__ __forceinline__ void put(double* slot) const {
+  __device__ __forceinline__ void put(double* slot, int warp) const {
     ff a;
     a.hi = s;
     a.lo = -c;
     a = warp_tree(a);
     if ((threadIdx.x & 31) == 0)
-      reinterpret_cast<float2*>(slot)[threadIdx.x >> 5] = make_float2(a.hi, a.lo);
+      reinterpret_cast<float2*>(slot)[warp] = make_float2(a.hi, a.lo);
   }
   static __device__ __forceinline__ double cross(const double* slot) {
     const int lane = threadIdx.x & 31;
@@ -1635,9 +1635,9 @@ struct AccD {  // Neumaier
     s = t;
   }
   __device__ __forceinline__ double value() const { return s + c; }
-  __device__ __forceinline__ void put(double* slot) const {
+  __device__ __forceinline__ void put(double* slot, int warp) const {
     const double x = warp_sum(value());
-    if ((threadIdx.x & 31) == 0) slot[threadIdx.x >> 5] = x;
+    if ((threadIdx.x & 31) == 0) slot[warp] = x;
   }
   static __device__ __forceinline__ double cross(const double* slot) {
     const int lane = threadIdx.x & 31;
@@ -1682,36 +1682,63 @@ template <typename T, bool CHI2> struct PointGroup {
   }
 };
 
+// Blocks (partial sums) of a chi-square over M points: at most `grid`, and no
+// more than have a group of points for every thread.  A block with few of its
+// threads at work costs its window copy, its reduction and its arrival all the
+// same: 64 cube channels of 1e5 to 1e6 points 416 -> 400 us (whole calls).
+//
+// A double point costs an SM's FP64 pipe 8 clocks, so few points want many SMs
+// rather than full blocks: 128 groups to a block.  (Whole calls in double, groups
+// for all 1024 or 256 threads, and 128, 64 and 32 groups to a block: side 64,
+// window in shared memory, 1e4 points 33.4, 24.6, 24.6, 25.5 us, 1e5 points 33.6,
+// 28.6, 28.7, 28.7 us; side 256, window through L2, 1e4 points 26.4, 24.5, 24.3,
+// 26.3 us, 1e5 points 28.9, 28.8, 30.0, 30.2 us.  With one copy of the body, in
+// gather_points, 128 groups: 22.6, 26.7, 22.6 and 26.7 us.)
+template <typename T> constexpr bool gather_few_groups() { return sizeof(T) == 8; }
+template <typename T> int gather_vblocks(int grid, int64_t M, int vec, int threads) {
+  const int64_t groups = vec ? M / Vec16<T>::W : M;
+  const int64_t per = gather_few_groups<T>() && threads > 128 ? 128 : threads;
+  const int64_t need = (groups + per - 1) / per;
+  return need < 1 ? 1 : need < grid ? (int)need : grid;
+}
+
 // Grid-stride layout of the vector groups: whole rounds of gstride groups,
 // then the remainder in equal contiguous slices, one per block (coalesced,
 // and no few blocks run a round more than the rest).
-// nblk blocks; at(bid): this thread in block bid (the divisions are done once,
-// 64-bit ones cost about as much as a point).
-struct GroupSplit {
+// Single calls: this thread of this block of the grid; BATCH: thread at_t of
+// virtual block at_bid, set by at(), of nblk (the divisions are done once, 64-bit
+// ones cost about as much as a point).
+template <bool BATCH> struct GroupSplit {
   int64_t nq, gstride, rounds, slice, rem_q, gtid;
+  int at_t, at_bid;
   __device__ __forceinline__ GroupSplit(int64_t M, int W, int vec, int nblk) {
     nq = vec ? M / W : 0;
     gstride = (int64_t)nblk * blockDim.x;
     rounds = nq / gstride;
     const int64_t rem = nq - rounds * gstride;
     slice = (rem + nblk - 1) / nblk;  // <= blockDim.x
+    at(blockIdx.x, threadIdx.x);
   }
-  __device__ __forceinline__ void at(int bid) {
-    rem_q = rounds * gstride + (int64_t)bid * slice + threadIdx.x;
-    gtid = (int64_t)bid * blockDim.x + threadIdx.x;
+  __device__ __forceinline__ void at(int bid_, int t_) {
+    at_t = t_;
+    at_bid = bid_;
+    rem_q = rounds * gstride + (int64_t)bid_ * slice + t_;
+    gtid = (int64_t)bid_ * blockDim.x + t_;
   }
-  __device__ __forceinline__ bool has_rem() const { return threadIdx.x < slice && rem_q < nq; }
+  __device__ __forceinline__ int t() const { return BATCH ? at_t : (int)threadIdx.x; }
+  __device__ __forceinline__ int bid() const { return BATCH ? at_bid : (int)blockIdx.x; }
+  __device__ __forceinline__ bool has_rem() const { return t() < slice && rem_q < nq; }
 };
 
 // pre: this thread's first group, already loaded by the caller, or null.
-template <typename T, bool CHI2, bool SMEM, bool EDGE, bool MULTI, bool FULL, typename ACC>
+template <typename T, bool CHI2, bool SMEM, bool EDGE, bool MULTI, bool FULL, typename ACC, bool BATCH>
 __device__ __forceinline__ void gather_points(const cplx_t<T>* __restrict__ G, const Window& win,
                                               const GatherT<T>& p, const T* __restrict__ u,
                                               const T* __restrict__ v, const T* __restrict__ re,
                                               const T* __restrict__ im, const T* __restrict__ w,
                                               int64_t M, int vec, cplx_t<T>* __restrict__ vis,
                                               ACC& acc, const MultiPhase<T>* mp,
-                                              const PointGroup<T, CHI2>* pre, const GroupSplit& sp,
+                                              const PointGroup<T, CHI2>* pre, const GroupSplit<BATCH>& sp,
                                               const fxtw* tab) {
   using C = cplx_t<T>;
   constexpr int W = Vec16<T>::W;
@@ -1749,21 +1776,40 @@ __device__ __forceinline__ void gather_points(const cplx_t<T>* __restrict__ G, c
       for (int e = 0; e < W; ++e) vis[q * W + e] = Vs[e];
     }
   };
-  auto group = [&](int64_t q) {
-    PointGroup<T, CHI2> g;
-    g.load(u, v, re, im, w, q);
-    compute(g, q);
-  };
   int64_t q = gtid;
   int64_t r = 0;
-  if (pre) {
-    compute(*pre, q);
-    q += sp.gstride;
-    r = 1;
+  if constexpr (sizeof(T) == 8) {
+    // one copy of the long body of a group: the kernel's three were 94 KB of
+    // instructions, which a short call waits for (256 image, 1e4 points 24.4 -> 22.6
+    // us; 4096^2 image, 5e6 points 283.5 -> 277.2 us)
+    PointGroup<T, CHI2> g;
+    bool here = pre != nullptr;
+    if (here) g = *pre;
+#pragma unroll 1
+    for (; r <= sp.rounds; ++r, q += sp.gstride) {
+      if (r == sp.rounds) {
+        if (!sp.has_rem()) break;
+        q = sp.rem_q;
+      }
+      if (!here) g.load(u, v, re, im, w, q);
+      here = false;
+      compute(g, q);
+    }
+  } else {
+    auto group = [&](int64_t q) {
+      PointGroup<T, CHI2> g;
+      g.load(u, v, re, im, w, q);
+      compute(g, q);
+    };
+    if (pre) {
+      compute(*pre, q);
+      q += sp.gstride;
+      r = 1;
+    }
+    for (; r < sp.rounds; ++r, q += sp.gstride) group(q);
+    if (sp.has_rem()) group(sp.rem_q);
   }
-  for (; r < sp.rounds; ++r, q += sp.gstride) group(q);
-  if (sp.has_rem()) group(sp.rem_q);
-  for (int64_t k = sp.nq * W + gtid; k < M; k += sp.gstride) {
+  auto single = [&](int64_t k) {
     const C V = point(u[k], v[k]);
     if constexpr (CHI2) {
       const T dr = re[k] - V.x, di = im[k] - V.y;
@@ -1771,18 +1817,18 @@ __device__ __forceinline__ void gather_points(const cplx_t<T>* __restrict__ G, c
     } else {
       vis[k] = V;
     }
+  };
+  if constexpr (gather_few_groups<T>()) {  // the points behind the groups, or all of them: as the groups
+    const int nblk = BATCH ? (int)(sp.gstride / blockDim.x) : (int)gridDim.x;
+    for (int64_t k0 = sp.nq * W; k0 < M; k0 += sp.gstride) {
+      const int64_t left = M - k0;
+      const int per = left < sp.gstride ? ((int)left + nblk - 1) / nblk : (int)blockDim.x;
+      const int64_t k = k0 + (int64_t)sp.bid() * per + sp.t();
+      if (sp.t() < per && k < M) single(k);
+    }
+  } else {
+    for (int64_t k = sp.nq * W + gtid; k < M; k += sp.gstride) single(k);
   }
-}
-
-// Blocks (partial sums) of a chi-square over M points: at most `grid`, and no
-// more than have a group of points for every thread.  A block with few of its
-// threads at work costs its window copy, its reduction and its arrival all the
-// same: 64 cube channels of 1e5 to 1e6 points 416 -> 400 us, a double image of 256
-// with 1e4 points 28.7 -> 26.4 us (whole calls).
-template <typename T> int gather_vblocks(int grid, int64_t M, int vec, int threads) {
-  const int64_t groups = vec ? M / Vec16<T>::W : M;
-  const int64_t need = (groups + threads - 1) / threads;
-  return need < 1 ? 1 : need < grid ? (int)need : grid;
 }
 
 // block shape: 512-thread blocks, two per SM, when the window is staged in
@@ -1838,8 +1884,7 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
   // 256 image with 1e4 points, but the selected address made 4096 / 5e6 3 % slower.)
   // (Single calls only: batched launches are not dependents.)
   constexpr int W = Vec16<T>::W;
-  GroupSplit gs(M, W, vec, nvb);
-  gs.at(blockIdx.x);
+  GroupSplit<(K > 1)> gs(M, W, vec, nvb);
   PointGroup<T, CHI2> g0;
   const bool pre = K == 1 && gs.rounds > 0;  // uniform over the grid
   if constexpr (K == 1) {
@@ -1913,13 +1958,15 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
       gather_points<T, CHI2, false, EDGE, MULTI, FULL>(Gw, win, p, u, v, re, im, w, M, vec, vis,
                                                        acc, mp, g0p, gs, tab);
     }
-    if constexpr (CHI2) acc.put(slot);
+    if constexpr (CHI2) acc.put(slot, gs.t() >> 5);
   };
   // The warps of a batched block run through its virtual blocks without waiting
   // for one another: each virtual block has its slot, and one barrier at the end
   // precedes the sums over warps, which the warps share out (two barriers and
   // three 64-bit divisions to each virtual block before: 64 walkers 1024 / 1e6
-  // 624 -> 573 us, 64 cube channels 379 -> 369 us).
+  // 624 -> 573 us, 64 cube channels 379 -> 369 us).  Where the points of a virtual
+  // block fill a part of its warps only (gather_vblocks), the next one begins at the
+  // next warps, so that a block works on all of them at once.
   constexpr int kSlots = K == 1 ? 1 : kMaxGatherFold;
   __shared__ double red[kSlots][32];
   if constexpr (K == 1) {
@@ -1932,11 +1979,18 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
       }
     }
   } else {
+    unsigned few = 0;  // threads that the points of a virtual block fill, where not all (whole warps)
+    if constexpr (gather_few_groups<T>()) {
+      const int64_t most = vec ? gs.slice : (M + nvb - 1) / nvb;
+      if (gs.rounds == 0 && most < blockDim.x) few = ((unsigned)most + 31u) & ~31u;
+    }
     for (int vb = blockIdx.x; vb < nvb;) {
       int n = 0, next = vb;
+      unsigned first = 0;  // thread that is thread 0 of the virtual block
       for (; n < kSlots && next < nvb; ++n, next += gridDim.x) {
-        gs.at(next);
+        gs.at(next, (int)((threadIdx.x - first) & (blockDim.x - 1)));
         run(nullptr, red[n]);
+        if constexpr (gather_few_groups<T>()) first += few;
       }
       __syncthreads();
       for (int k = threadIdx.x >> 5; k < n; k += (int)(blockDim.x >> 5)) {
