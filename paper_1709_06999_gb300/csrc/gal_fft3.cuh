@@ -64,16 +64,18 @@ template <typename T, int V> struct TwTab {
   static __host__ __device__ constexpr size_t fx_col(int N) { return (size_t)3 * N; }
   static __host__ __device__ constexpr size_t fx_row(int N) { return (size_t)4 * N; }
 };
-// entry i of the staged table of length L at radix V: its exponent in units of 1/L turns
-__host__ __device__ inline int tw_stage_exponent(int L, int V, int i) {
-  int Ns = V, R = V;  // span and radix of the stage
+// entry i of the staged table of length L = 2^lg at radix V = 2^lv: its exponent in
+// units of 1/L turns
+__host__ __device__ inline int tw_stage_exponent(int lg, int lv, int i) {
+  int ns = lv, r = lv;  // span and radix of the stage, log2
   for (;;) {
-    if (Ns * V >= L) R = L / Ns;
-    if (i < (R - 1) * Ns) break;
-    i -= (R - 1) * Ns;
-    Ns *= V;
+    if (ns + lv >= lg) r = lg - ns;
+    const int n = ((1 << r) - 1) << ns;  // its entries
+    if (i < n) break;
+    i -= n;
+    ns += lv;
   }
-  return (i / Ns + 1) * (i % Ns) * (L / (Ns * R));
+  return (((i >> ns) + 1) * (i & ((1 << ns) - 1))) << (lg - ns - r);
 }
 
 template <int V> __device__ __forceinline__ int pad3(int a) { return a + (a >> ilog2c(V)); }
