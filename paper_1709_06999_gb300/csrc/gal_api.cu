@@ -37,6 +37,15 @@ struct TimedStage {
 
 }  // namespace
 
+// What a registration's extent pass needs: its state (Launch::extent) and a result
+// in mapped host memory.
+struct RegSlot {
+  void* state = nullptr;
+  double* rho2 = nullptr;
+  RegSlot* next = nullptr;
+};
+constexpr int kRegSlots = 64;
+
 struct gal_ctx {
   int device = 0;
   int num_sms = 0;
@@ -48,11 +57,15 @@ struct gal_ctx {
   int partials_len = 0;
   unsigned* counter = nullptr;  // last-block-done counter (self-resetting)
   double* rho2 = nullptr;       // uv extent scratch for raw-pointer calls
-  void* ext_state = nullptr;    // Launch::extent's: of those calls, and of registrations
-  // registrations (a server's may come from several threads at once): the extent of
-  // the one that holds reg_mu, in mapped host memory
-  std::mutex reg_mu;
-  double* reg_rho2 = nullptr;
+  void* ext_state = nullptr;    // Launch::extent's: of those calls, then of reg_first's slots
+  // Registrations may come from several threads at once, on different streams: each
+  // takes a slot and gives it back when its extent is read.  The first kRegSlots are
+  // made with the context, more when all are in use (pinned memory allocated then
+  // would wait for the device).
+  std::mutex reg_mu;             // of the list of free slots only
+  RegSlot* reg_free = nullptr;
+  RegSlot reg_first[kRegSlots];
+  double* reg_rho2 = nullptr;    // mapped host memory of reg_first
   double* uvrange = nullptr;    // min / max of u^2 + v^2 (image sizing)
   int* err = nullptr;           // index-check flag
   double* chi2_dev = nullptr;   // result slot for the host-buffer entry points
@@ -583,6 +596,36 @@ int sweep_t(gal_ctx* ctx, const T* I, int nr, double Rmin, double dR, int nxy, d
   });
 }
 
+// A free registration slot; a new one's state is cleared on `st`, whose extent pass
+// is its first user.
+int take_reg_slot(gal_ctx* ctx, cudaStream_t st, RegSlot** out) {
+  {
+    std::lock_guard<std::mutex> lk(ctx->reg_mu);
+    if (RegSlot* r = ctx->reg_free) {
+      ctx->reg_free = r->next;
+      *out = r;
+      return GAL_OK;
+    }
+  }
+  RegSlot* r = new (std::nothrow) RegSlot;
+  if (!r) return GAL_E_NOMEM;
+  cudaError_t e = cudaMalloc(&r->state, gal::kExtentState);
+  if (!e) e = cudaMemsetAsync(r->state, 0, gal::kExtentState, st);
+  if (!e) e = cudaHostAlloc((void**)&r->rho2, sizeof(double), cudaHostAllocMapped);
+  if (e) {
+    if (r->state) cudaFree(r->state);
+    delete r;
+    return cuda_fail(ctx, e);
+  }
+  *out = r;
+  return GAL_OK;
+}
+void give_reg_slot(gal_ctx* ctx, RegSlot* r) {
+  std::lock_guard<std::mutex> lk(ctx->reg_mu);
+  r->next = ctx->reg_free;
+  ctx->reg_free = r;
+}
+
 template <typename T>
 int data_create_t(gal_ctx* ctx, const T* u, const T* v, const T* re, const T* im, const T* w,
                   int64_t M, void* stream, gal_data** out) {
@@ -606,21 +649,23 @@ int data_create_t(gal_ctx* ctx, const T* u, const T* v, const T* re, const T* im
     // the extent comes back once, into mapped host memory: every call sizes its
     // window from it on the host and passes the kernels the result
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    std::lock_guard<std::mutex> lk(ctx->reg_mu);  // until the extent is read
-    int s = stage(ctx, 0, st, [&] {
-      return gal::Launch<T>::extent(u, v, M, ctx->reg_rho2,
-                                    static_cast<char*>(ctx->ext_state) + gal::kExtentState,
-                                    ctx->num_sms, st);
-    });
+    RegSlot* slot = nullptr;
+    int s = take_reg_slot(ctx, st, &slot);
     if (s == GAL_OK) {
-      const cudaError_t e = cudaStreamSynchronize(st);
-      if (e != cudaSuccess) s = cuda_fail(ctx, e);
+      s = stage(ctx, 0, st, [&] {
+        return gal::Launch<T>::extent(u, v, M, slot->rho2, slot->state, ctx->num_sms, st);
+      });
+      if (s == GAL_OK) {
+        const cudaError_t e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) s = cuda_fail(ctx, e);
+      }
+      d->rho2_host = *static_cast<volatile double*>(slot->rho2);
+      give_reg_slot(ctx, slot);
     }
     if (s != GAL_OK) {
       delete d;
       return s;
     }
-    d->rho2_host = *static_cast<volatile double*>(ctx->reg_rho2);
   }
   *out = d;
   return GAL_OK;
@@ -1245,9 +1290,15 @@ int gal_create(gal_ctx** out, int device) {
   if (!e) e = cudaMalloc(&ctx->partials, sizeof(double) * (size_t)maxb);
   if (!e) e = cudaMalloc(&ctx->counter, sizeof(unsigned));
   if (!e) e = cudaMalloc(&ctx->rho2, sizeof(double));
-  if (!e) e = cudaMalloc(&ctx->ext_state, 2 * gal::kExtentState);
-  if (!e) e = cudaMemset(ctx->ext_state, 0, 2 * gal::kExtentState);
-  if (!e) e = cudaHostAlloc((void**)&ctx->reg_rho2, sizeof(double), cudaHostAllocMapped);
+  if (!e) e = cudaMalloc(&ctx->ext_state, (1 + kRegSlots) * gal::kExtentState);
+  if (!e) e = cudaMemset(ctx->ext_state, 0, (1 + kRegSlots) * gal::kExtentState);
+  if (!e) e = cudaHostAlloc((void**)&ctx->reg_rho2, kRegSlots * sizeof(double), cudaHostAllocMapped);
+  if (!e)
+    for (int k = 0; k < kRegSlots; ++k) {
+      ctx->reg_first[k].state = static_cast<char*>(ctx->ext_state) + (1 + k) * gal::kExtentState;
+      ctx->reg_first[k].rho2 = ctx->reg_rho2 + k;
+      give_reg_slot(ctx, &ctx->reg_first[k]);
+    }
   if (!e) e = cudaMalloc(&ctx->uvrange, 2 * sizeof(double));
   if (!e) e = cudaMalloc(&ctx->err, sizeof(int));
   if (!e) e = cudaMalloc(&ctx->chi2_dev, sizeof(double));
@@ -1272,6 +1323,15 @@ void gal_destroy(gal_ctx* ctx) {
                   (void*)ctx->err, (void*)ctx->chi2_dev, ctx->stage_img, ctx->beam,
                   ctx->pipe_img[0], ctx->pipe_img[1], (void*)ctx->pipe_chi2})
     if (p) cudaFree(p);
+  for (RegSlot* r = ctx->reg_free; r;) {
+    RegSlot* next = r->next;
+    if (r < ctx->reg_first || r >= ctx->reg_first + kRegSlots) {
+      cudaFree(r->state);
+      cudaFreeHost(r->rho2);
+      delete r;
+    }
+    r = next;
+  }
   if (ctx->reg_rho2) cudaFreeHost(ctx->reg_rho2);
   for (cudaEvent_t e : {ctx->pipe_copied[0], ctx->pipe_copied[1], ctx->pipe_done[0],
                         ctx->pipe_done[1]})
