@@ -29,10 +29,6 @@ template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
 // a * (-i)
 template <typename C> __device__ __forceinline__ C cmul_mi(C a) { return mkc(a.y, -a.x); }
 template <typename C> __device__ __forceinline__ C cconj(C a) { return mkc(a.x, -a.y); }
-// a + f (b - a), componentwise
-template <typename C, typename T> __device__ __forceinline__ C clerp(C a, C b, T f) {
-  return mkc(a.x + f * (b.x - a.x), a.y + f * (b.y - a.y));
-}
 
 // ---------------------------------------------------------------------------
 // float-float arithmetic: a value is hi + lo with |lo| <= ulp(hi)/2, about 48

@@ -300,24 +300,20 @@ __device__ __forceinline__ void sweep_row(cplx_t<T> (&z)[V], const T* __restrict
                                           const SweepT<T>& sp, int row, int t, T* xs, bool act) {
   constexpr int N = 2 * M, TT = M / V;
   const int irow = (row + M) & (N - 1);
-  if constexpr (V < 2) {
-    z[0] = mkc((T)0, (T)0);
-  } else {
-    if (act) {
+  if (act) {
 #pragma unroll
-      for (int r = 0; r < V / 2; ++r) {
-        const int m = t + r * TT;  // shifted columns 2 m < N/2: image columns 2 m + N/2
-        z[r] = mkc(sweep_pixel(I, sp, N, irow, 2 * m + M), sweep_pixel(I, sp, N, irow, 2 * m + 1 + M));
-        reinterpret_cast<cplx_t<T>*>(xs)[m] = z[r];
-      }
-      if (t == 0) xs[M] = sweep_pixel(I, sp, N, irow, 0);
+    for (int r = 0; r < V / 2; ++r) {
+      const int m = t + r * TT;  // shifted columns 2 m < N/2: image columns 2 m + N/2
+      z[r] = mkc(sweep_pixel(I, sp, N, irow, 2 * m + M), sweep_pixel(I, sp, N, irow, 2 * m + 1 + M));
+      reinterpret_cast<cplx_t<T>*>(xs)[m] = z[r];
     }
-    __syncthreads();
+    if (t == 0) xs[M] = sweep_pixel(I, sp, N, irow, 0);
+  }
+  __syncthreads();
 #pragma unroll
-    for (int r = V / 2; r < V; ++r) {
-      const int m = t + r * TT;
-      z[r] = act ? mkc(xs[N - 2 * m], xs[N - 2 * m - 1]) : mkc((T)0, (T)0);
-    }
+  for (int r = V / 2; r < V; ++r) {
+    const int m = t + r * TT;
+    z[r] = act ? mkc(xs[N - 2 * m], xs[N - 2 * m - 1]) : mkc((T)0, (T)0);
   }
 }
 
