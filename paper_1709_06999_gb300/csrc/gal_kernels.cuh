@@ -2124,7 +2124,7 @@ inline int col_threads_per_col(int N) { return N >= 8 ? N / 8 : 1; }
 
 // Resident blocks per SM of a kernel that is always launched with the same block
 // and shared memory, at least 1 (asked once per device: the query takes most of a
-// microsecond on the host).
+// microsecond on the host; a query that fails is asked again).
 template <auto Kern> int resident_blocks(int threads, size_t smem) {
   static std::atomic<int> cache[64] = {};
   int d = 0, n = 0;
@@ -2132,7 +2132,7 @@ template <auto Kern> int resident_blocks(int threads, size_t smem) {
   n = cache[d].load(std::memory_order_relaxed);
   if (!n) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, Kern, threads, smem) != cudaSuccess || n < 1)
-      n = 1;
+      return 1;
     cache[d].store(n, std::memory_order_relaxed);
   }
   return n;
