@@ -40,7 +40,10 @@ __global__ void __launch_bounds__(FxRowShape<LG>::SH::threads,
                                   min_blocks_128regs<FxRowShape<LG>::SH::threads>())
 row_fx_kernel(const __grid_constant__ Jobs<RowJob<double>, K> jobs, const double2* __restrict__ twd,
               int* __restrict__ err) {
-  grid_dep_launch();  // the column pass may be scheduled as our blocks retire
+  // The column pass may be scheduled as our blocks retire.  No wait comes first, and
+  // the image is read before one: this kernel is launched normally or after a kernel
+  // that is (see launch_dependent).
+  grid_dep_launch();
   using S = FxRowShape<LG>;
   using SH = typename S::SH;
   using P = typename SH::P;

@@ -129,9 +129,12 @@ constexpr int kBatchJobs = 32;
 constexpr int kAltRadix = 8;
 constexpr int kAltRadixMaxSide = 512;
 // Default plan.  Short float columns run at radix 8: twice the threads to a
-// column (side 512: 27 against 33 us for 32 unpruned images in a batch, 7.8
-// against 10.9 for one; level or better down to 32 but for batches of side 256,
-// 12.9 against 10.9).  Rows run at radix 8 where it takes no more stages than
+// column (whole calls with an almost complete window, radix 8 against 16, one image
+// and batches of 4 and 32: side 512 11.4, 26.5, 57.5 against 14.8, 28.9, 64.4 us;
+// 256 11.4, 23.8, 29.0 against 12.0, 24.8, 29.0; 128 11.2, 24.8, 26.8 against 11.7,
+// 24.8, 26.5; 64 11.1, 22.8, 26.8 against 11.8, 24.8, 26.5; 32 10.9, 22.7, 26.1
+// against 11.4, 22.7, 26.2.  With a tenth of the window, 32 images of side 512 take
+// 35.1 against 33.7 us, everything else is level or better).  Rows run at radix 8 where it takes no more stages than
 // radix 16, i.e. for 32 and 64 complex points, sides 64 and 128 (12.0 against
 // 14.2 and 11.8 against 14.1 us for 32 images), and at 16 elsewhere (side 512:
 // 23 against 28 us).  A rule, not a timing in each process, because the two

@@ -2083,6 +2083,15 @@ template <typename T, auto Kern> cudaError_t ensure_l1_carveout() {
 // Launch `kern` as a programmatic dependent of the preceding kernel in `st`:
 // it may be scheduled while that kernel finishes, and waits for it in
 // grid_dep_wait() before reading what it wrote.
+//
+// Several kernels read before they wait: the gather its first points, the double
+// row pass and those with a beam their image, all of them their factors.  That is
+// sound only because these are inputs of the call, and because the first kernel of
+// a chain (extent pass, beam tables, or the row pass) is either launched normally or
+// waits before it triggers its dependents: everything enqueued before the call is
+// then complete when any later kernel of the chain starts.  A row pass that is to
+// follow the previous call's gather must therefore wait before its trigger and
+// before its first read.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                              cudaStream_t st, Args&&... args) {
