@@ -44,7 +44,7 @@ struct RegSlot {
   double* rho2 = nullptr;
   RegSlot* next = nullptr;
 };
-constexpr int kRegSlots = 64;
+constexpr int kRegSlots = 31;  // with the state of raw-pointer calls 512 bytes
 
 struct gal_ctx {
   int device = 0;
