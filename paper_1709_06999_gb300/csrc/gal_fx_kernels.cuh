@@ -2,9 +2,10 @@
 // (gal_fx.cuh): the passes of gal_kernels.cuh with each sequence brought to a
 // common power of two before its transform.  Images, F1 and the window are
 // doubles.  Measured against the same passes in FP64 arithmetic (which kept the
-// FP64 pipe 83 % busy): row pass of 4096^2 pixels, 61 columns kept, 481 -> 113
-// us (now 100); of 2048^2 pixels, 413 columns kept, 161 -> 38 us; column pass of 4096 x 61
-// 41 -> 12 us, of 2048 x 413 66 -> 19 us.
+// FP64 pipe 83 % busy): row pass of 4096^2 pixels, 61 columns kept, 481 -> 102
+// us; of 2048^2 pixels, 413 columns kept, 161 -> 39 us; column pass of 4096 x 61
+// 41 -> 12 us, of 2048 x 413 66 -> 19 us.  (With one scale for all stages, which
+// lost precision, the row passes took 100 and 38 us.)
 #pragma once
 
 #include "gal_fx.cuh"

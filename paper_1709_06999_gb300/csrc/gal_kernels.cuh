@@ -1505,8 +1505,8 @@ __device__ __forceinline__ void sample_pair(const float2* __restrict__ G, const 
 // double path: FP64 for the rotation and the phase argument, integers (gal_fx.cuh)
 // for the cell, the interpolation, the sine and cosine and the phase rotation:
 // about 17 FP64 instructions a point instead of about 95, which bounded this
-// kernel (5e6 points, window in shared memory: 726 -> 168 us; 1e6 points, window
-// through L2: 155 -> 48 us).  tab: the sine / cosine table in shared memory.
+// kernel (5e6 points, window in shared memory: 726 -> 164 us; 1e6 points, window
+// through L2: 155 -> 47 us).  tab: the sine / cosine table in shared memory.
 template <bool SMEM, bool EDGE, bool MULTI = false, bool FULL = false>
 __device__ __forceinline__ double2 sample_point(const cplx_t<double>* __restrict__ Gp, const Window& w,
                                                 const GatherT<double>& p, double u, double v,
@@ -1704,10 +1704,10 @@ template <typename T> int gather_vblocks(int grid, int64_t M, int vec, int threa
 // Grid-stride layout of the vector groups: whole rounds of gstride groups,
 // then the remainder in equal contiguous slices, one per block (coalesced,
 // and no few blocks run a round more than the rest).
-// Single calls: this thread of this block of the grid; BATCH: thread at_t of
-// virtual block at_bid, set by at(), of nblk (the divisions are done once, 64-bit
-// ones cost about as much as a point).
-template <bool BATCH> struct GroupSplit {
+// nblk blocks; at(): this thread in (virtual) block bid (the divisions are done once,
+// 64-bit ones cost about as much as a point).  MOVED: as its thread t, which need not
+// be threadIdx.x (double batches; float ones lose 1 % with a variable t).
+template <bool MOVED> struct GroupSplit {
   int64_t nq, gstride, rounds, slice, rem_q, gtid;
   int at_t, at_bid;
   __device__ __forceinline__ GroupSplit(int64_t M, int W, int vec, int nblk) {
@@ -1724,20 +1724,20 @@ template <bool BATCH> struct GroupSplit {
     rem_q = rounds * gstride + (int64_t)bid_ * slice + t_;
     gtid = (int64_t)bid_ * blockDim.x + t_;
   }
-  __device__ __forceinline__ int t() const { return BATCH ? at_t : (int)threadIdx.x; }
-  __device__ __forceinline__ int bid() const { return BATCH ? at_bid : (int)blockIdx.x; }
+  __device__ __forceinline__ int t() const { return MOVED ? at_t : (int)threadIdx.x; }
+  __device__ __forceinline__ int bid() const { return MOVED ? at_bid : (int)blockIdx.x; }
   __device__ __forceinline__ bool has_rem() const { return t() < slice && rem_q < nq; }
 };
 
 // pre: this thread's first group, already loaded by the caller, or null.
-template <typename T, bool CHI2, bool SMEM, bool EDGE, bool MULTI, bool FULL, typename ACC, bool BATCH>
+template <typename T, bool CHI2, bool SMEM, bool EDGE, bool MULTI, bool FULL, typename ACC, bool MOVED>
 __device__ __forceinline__ void gather_points(const cplx_t<T>* __restrict__ G, const Window& win,
                                               const GatherT<T>& p, const T* __restrict__ u,
                                               const T* __restrict__ v, const T* __restrict__ re,
                                               const T* __restrict__ im, const T* __restrict__ w,
                                               int64_t M, int vec, cplx_t<T>* __restrict__ vis,
                                               ACC& acc, const MultiPhase<T>* mp,
-                                              const PointGroup<T, CHI2>* pre, const GroupSplit<BATCH>& sp,
+                                              const PointGroup<T, CHI2>* pre, const GroupSplit<MOVED>& sp,
                                               const fxtw* tab) {
   using C = cplx_t<T>;
   constexpr int W = Vec16<T>::W;
@@ -1818,7 +1818,7 @@ __device__ __forceinline__ void gather_points(const cplx_t<T>* __restrict__ G, c
     }
   };
   if constexpr (gather_few_groups<T>()) {  // the points behind the groups, or all of them: as the groups
-    const int nblk = BATCH ? (int)(sp.gstride / blockDim.x) : (int)gridDim.x;
+    const int nblk = MOVED ? (int)(sp.gstride / blockDim.x) : (int)gridDim.x;
     for (int64_t k0 = sp.nq * W; k0 < M; k0 += sp.gstride) {
       const int64_t left = M - k0;
       const int per = left < sp.gstride ? ((int)left + nblk - 1) / nblk : (int)blockDim.x;
@@ -1883,7 +1883,8 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
   // 256 image with 1e4 points, but the selected address made 4096 / 5e6 3 % slower.)
   // (Single calls only: batched launches are not dependents.)
   constexpr int W = Vec16<T>::W;
-  GroupSplit<(K > 1)> gs(M, W, vec, nvb);
+  constexpr bool MOVED = K > 1 && gather_few_groups<T>();
+  GroupSplit<MOVED> gs(M, W, vec, nvb);
   PointGroup<T, CHI2> g0;
   const bool pre = K == 1 && gs.rounds > 0;  // uniform over the grid
   if constexpr (K == 1) {
@@ -1979,7 +1980,7 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
     }
   } else {
     unsigned few = 0;  // threads that the points of a virtual block fill, where not all (whole warps)
-    if constexpr (gather_few_groups<T>()) {
+    if constexpr (MOVED) {
       const int64_t most = vec ? gs.slice : (M + nvb - 1) / nvb;
       if (gs.rounds == 0 && most < blockDim.x) few = ((unsigned)most + 31u) & ~31u;
     }
@@ -1987,9 +1988,9 @@ gather_kernel(const __grid_constant__ Jobs<GatherJob<T>, K> jobs, int smem_nodes
       int n = 0, next = vb;
       unsigned first = 0;  // thread that is thread 0 of the virtual block
       for (; n < kSlots && next < nvb; ++n, next += gridDim.x) {
-        gs.at(next, (int)((threadIdx.x - first) & (blockDim.x - 1)));
+        gs.at(next, MOVED ? (int)((threadIdx.x - first) & (blockDim.x - 1)) : (int)threadIdx.x);
         run(nullptr, red[n]);
-        if constexpr (gather_few_groups<T>()) first += few;
+        if constexpr (MOVED) first += few;
       }
       __syncthreads();
       for (int k = threadIdx.x >> 5; k < n; k += (int)(blockDim.x >> 5)) {
