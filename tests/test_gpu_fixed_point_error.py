@@ -61,3 +61,28 @@ def test_error_is_that_of_double_arithmetic(kind, n):
     dr, di = got[:, 0] - re.ravel(), got[:, 1] - im.ravel()
     err = math.sqrt(float(np.sum(dr * dr + di * di) / np.sum(re * re + im * im)))
     assert err <= 2.0 ** -53 * math.sqrt(2 * math.log2(n)), err
+
+
+@pytest.mark.parametrize("n", [64, 128, 256, 512, 1024, 2048, 4096, 8192])
+def test_sums_as_large_as_they_can_be(n):
+    """Images whose values add up without cancelling, in every stage: the bound that
+    the integers are scaled to is reached, and none of them may wrap."""
+    ctx = Context(0)
+    dxy = 2.0 ** -27
+    k, l = np.meshgrid(np.arange(K + 1), np.arange(-K, K + 1))
+    u, v = (torch.as_tensor(a.ravel() / (n * dxy), device="cuda") for a in (k, l))
+    i = np.arange(n)
+    ones = np.ones((n, n))
+    wave = np.cos(2 * np.pi * ((3 * i[:, None] + 5 * i[None, :]) % n) / n)
+    corner = np.zeros((n, n))
+    corner[0] = corner[:, n // 4] = 1.0  # a full row and a full column
+    spike = np.rint(wave * 3)
+    spike[n // 3, n // 5] = 2.0 ** 20 - 1
+    for img in (ones * (2 ** 20 - 1), ones * 2 ** 19, np.rint(wave * (2 ** 20 - 1)),
+                np.where((i[:, None] + i[None, :]) % 2, -1.0, 1.0) * (2 ** 20 - 1),
+                corner * (2 ** 20 - 1), spike):
+        got = ctx.sample_image(torch.as_tensor(img, device="cuda"), dxy, u, v).cpu().numpy()
+        re, im = exact_nodes(img)
+        err = np.max(np.hypot(got[:, 0] - re.ravel(), got[:, 1] - im.ravel()).astype(np.float64))
+        # every level rounds at 2^-53 of the largest value the level can have
+        assert err <= 2 * math.log2(n) * 2.0 ** -53 * np.abs(img).sum()
